@@ -707,6 +707,17 @@ __global__ void k_sell_compact(Sell A, const int64_t* __restrict__ usize,
     if (lane == 0) A.ucptr[s] = o;
 }
 
+__global__ void k_sell_info(Sell A) {
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= A.nslices) return;
+    const int64_t base = A.sptr[s], up = A.ucptr[s];
+    int w = A.width[s];
+    if (up >= 0)
+        for (int k = A.width[s] - 1; k >= 0; --k)
+            if (A.ucode[up + k] & 1) w |= SINFO_ABS;
+    A.sinfo[s] = make_int4((int)(uint32_t)base, (int)(base >> 32), (int)up, w);
+}
+
 // Uniform slices that hold the same stencil (width, column codes and FP64 values
 // all equal) share one stored copy: on a lattice most interior slices carry the
 // same stencil, so the distinct stencils are few (the bumpy channel's Poisson
@@ -788,7 +799,12 @@ static vip_status sell_uniform(vip_ctx* c, Sell& S) {
     k_sell_compact<<<grid, TB, 0, st>>>(S, usize, uoff);
     VIP_CUDA(cudaGetLastError());
     VIP_CUDA(cudaStreamSynchronize(st));
-    return sell_share_stencils(c, S, hw);
+    vip_status sh = sell_share_stencils(c, S, hw);
+    if (sh != VIP_OK) return sh;
+    VIP_CUDA(dalloc(c, &S.sinfo, S.nslices));
+    k_sell_info<<<(unsigned)((S.nslices + TB - 1) / TB), TB, 0, st>>>(S);
+    VIP_CUDA(cudaGetLastError());
+    return VIP_OK;
 }
 
 static vip_status build_table(vip_ctx* c, const AsmArgs& A, int tb, int64_t nrows, Sell& S,

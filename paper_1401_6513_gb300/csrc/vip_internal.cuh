@@ -14,6 +14,7 @@ namespace vip {
 
 constexpr int SLICE = 32;           // SELL-C slice height = warp size
 constexpr int KMAX = 64;            // largest neighbour list per point
+constexpr int SINFO_WIDTH = 0xffff, SINFO_ABS = 1 << 16;  // fields of Sell::sinfo.w
 constexpr int NPTYPE = 7;           // point types: node, E, W, N, S, probe1, probe2
 enum PointType { PT_NODE = 0, PT_E = 1, PT_W = 2, PT_N = 3, PT_S = 4, PT_B1 = 5, PT_B2 = 6 };
 constexpr uint8_t KIND_PAD = 255;   // padding row (not a node)
@@ -52,6 +53,9 @@ struct Sell {
     int32_t* ucode = nullptr;     // [nuentries]
     double* uv64 = nullptr;
     float* uv32 = nullptr;
+    // one 16-byte record per slice: x, y = low and high word of sptr[s], z = ucptr[s] (-1:
+    // not uniform), w = width | SINFO_ABS if the shared stencil holds an absolute column
+    int4* sinfo = nullptr;        // [nslices] (Krylov operators only)
     int64_t nuniform = 0;         // uniform slices
     int64_t nuentries = 0;        // entries of their stored stencils (slices with the same
                                   // stencil share one copy)
@@ -87,7 +91,7 @@ struct GeomDev {
 constexpr int MAXSYS_PB = 16;   // systems a block may touch
 constexpr int NQ = 4;           // reduced quantities per phase
 struct KrylovPlan {
-    int nblocks = 0, nthreads = 0, nsys = 0;
+    int nblocks = 0, nsys = 0;
     int64_t nslices = 0;
     // device arrays
     int32_t* slice_sys = nullptr;   // [nslices] system of each slice

@@ -132,23 +132,23 @@ __global__ void k_mg_galerkin(int64_t nc, const int64_t* __restrict__ child,  //
 
 // sliced copy of the stencils ([n/32][25][32]), the l1-Jacobi scaling
 // -1 / sum_o |a_co| of the smoother (0 for empty and padding cells), and per
-// slice of 32 cells whether any stencil has a nonzero outside the central 3 x 3
-// offsets.  Away from boundaries a 2 x 2 aggregate of the 13-point fine stencil, and
+// slice of 32 cells the offsets outside the central 3 x 3 at which any stencil has a
+// nonzero.  Away from boundaries a 2 x 2 aggregate of the 13-point fine stencil, and
 // of a 3 x 3 coarse stencil, couples only to the adjacent cells, so most slices
 // need 9 of the 25 products.  n is a multiple of 32 and blockDim a multiple of 32,
 // so each warp is one slice.
 __global__ void k_mg_finish(int64_t n, const double* __restrict__ coef, double* __restrict__ coefs,
-                            double* __restrict__ dinv, uint8_t* __restrict__ ring) {
+                            double* __restrict__ dinv, uint32_t* __restrict__ ring) {
     int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n) return;
     double s = 0.0;
-    bool outer = false;
+    uint32_t outer = 0;
     for (int o = 0; o < 25; ++o) {
         const double a = coef[(int64_t)o * n + c];
         coefs[(c >> 5) * 800 + o * 32 + (c & 31)] = a;
         s += fabs(a);
         const int dy = o / 5 - 2, dx = o % 5 - 2;
-        if ((dx < -1 || dx > 1 || dy < -1 || dy > 1) && a != 0.0) outer = true;
+        if ((dx < -1 || dx > 1 || dy < -1 || dy > 1) && a != 0.0) outer |= 1u << o;
     }
     // Every row of the Poisson operator that reaches the coarse levels is a node
     // equation with a negative diagonal (Laplacian rows, and boundary rows scaled to
@@ -157,8 +157,8 @@ __global__ void k_mg_finish(int64_t n, const double* __restrict__ coef, double* 
     // diagonal would push the error the wrong way.  So the step has the operator's
     // sign on every cell.
     dinv[c] = (s != 0.0) ? -1.0 / s : 0.0;
-    const unsigned any = __ballot_sync(0xffffffffu, outer);
-    if ((threadIdx.x & 31) == 0) ring[c >> 5] = any ? 1 : 0;
+    const uint32_t any = __reduce_or_sync(0xffffffffu, outer);
+    if ((threadIdx.x & 31) == 0) ring[c >> 5] = any;
 }
 
 // fine-level l1-Jacobi scaling sign(a_rr) / sum_k |a_rk|
@@ -425,6 +425,15 @@ vip_status mg_build(vip_ctx* c, Multigrid& M) {
         std::vector<int64_t> cur(ptr.begin(), ptr.end() - 1);
         for (int64_t r = 0; r < R; ++r)
             if (agg[r] >= 0) rows[cur[agg[r]]++] = (int32_t)r;
+        std::vector<int4> rows4(n1);
+        for (int64_t i = 0; i < n1; ++i) {
+            const int64_t k = ptr[i + 1] - ptr[i];
+            const int32_t* q = rows.data() + ptr[i];
+            rows4[i] = make_int4(k > 0 ? q[0] : -1, k > 1 ? q[1] : -1, k > 2 ? q[2] : -1,
+                                 k > 4 ? -2 : k > 3 ? q[3] : -1);
+        }
+        VIP_CUDA(dalloc(c, &M.crow4, n1));
+        VIP_CUDA(cudaMemcpyAsync(M.crow4, rows4.data(), n1 * sizeof(int4), cudaMemcpyHostToDevice, st));
         VIP_CUDA(dalloc(c, &M.cptr, n1 + 1));
         VIP_CUDA(dalloc(c, &M.crow, rows.size()));
         VIP_CUDA(cudaMemcpyAsync(M.cptr, ptr.data(), (n1 + 1) * 8, cudaMemcpyHostToDevice, st));

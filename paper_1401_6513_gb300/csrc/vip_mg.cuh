@@ -2,6 +2,7 @@
 // (vip_mg.cu) and the V-cycle inside the Krylov launch (vip_krylov.cu).
 #pragma once
 
+#include <cuda_runtime.h>
 #include <stdint.h>
 
 namespace vip {
@@ -49,7 +50,7 @@ struct MgLevel {                  // coarse level (all geometries concatenated)
     double* dinv = nullptr;       // [n] l1-Jacobi scaling (0 for empty and padding cells)
     double* wdinv = nullptr;      // [n] omega * dinv (the smoother's step)
     float* wdinv32 = nullptr;     // [n] omega * dinv rounded to FP32
-    uint8_t* ring = nullptr;      // [n/32] 1 if a cell of the slice has a nonzero outside its 3 x 3 core
+    uint32_t* ring = nullptr;     // [n/32] bit o: a cell of the slice has a nonzero at outer offset o (of 25)
     MgLevGeom* lg = nullptr;      // [G] lattice of each geometry on this level
     MgTile* tiles = nullptr;      // 32 x th tiles covering every geometry's lattice
     int64_t ntiles = 0;
@@ -65,6 +66,7 @@ struct Multigrid {
     int32_t* agg = nullptr;       // [R] level-1 cell of a fine row (-1: none)
     int64_t* cptr = nullptr;      // [n1+1] fine rows of each level-1 cell
     int32_t* crow = nullptr;
+    int4* crow4 = nullptr;        // [n1] a level-1 cell's rows, ascending (-1: none); w = -2: more than four
     double* fdinv = nullptr;      // [R] l1-Jacobi scaling of the fine operator
     double* fwdinv = nullptr;     // [R] omega * fdinv
     float* fwdinv32 = nullptr;    // [R] omega * fdinv rounded to FP32
@@ -89,6 +91,7 @@ struct MgDev {
     const int32_t* agg;
     const int64_t* cptr;
     const int32_t* crow;
+    const int4* crow4;
     const T* fwdinv;        // omega * fine l1-Jacobi scaling
     T* fr;
     T* fx;
@@ -97,7 +100,7 @@ struct MgDev {
     const MgLevGeom* lg[MG_MAXLEV + 1];
     const MgTile* tiles[MG_MAXLEV + 1];
     const T* coefs[MG_MAXLEV + 1];            // sliced stencils
-    const uint8_t* ring[MG_MAXLEV + 1];       // slices whose stencils reach beyond 3 x 3
+    const uint32_t* ring[MG_MAXLEV + 1];      // outer offsets that the slices' stencils hold
     int32_t th[MG_MAXLEV + 1];                // tile heights
     const T* wdinv[MG_MAXLEV + 1];            // omega * l1-Jacobi scaling
     T* x[MG_MAXLEV + 1];
