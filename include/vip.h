@@ -616,8 +616,7 @@ vip_status vip_3d_apply(vip_3d* b, int which, const double* x, double* y);
  *   VIP_ERR_ARG the fields and the Adams-Bashforth history are partly updated:
  *   set the state again before stepping on.  Errors: VIP_ERR_ARG (not built, no
  *   flow or state, SLIP or OUTLET nodes, no interior node), VIP_ERR_NOT_CONVERGED,
- *   VIP_ERR_BREAKDOWN,
- *   VIP_ERR_NONFINITE, VIP_ERR_CUDA, VIP_ERR_OOM.
+ *   VIP_ERR_BREAKDOWN, VIP_ERR_NONFINITE, VIP_ERR_TIMEOUT, VIP_ERR_CUDA, VIP_ERR_OOM.
  * vip_3d_get_state: u, v, w, p, phi of every node into caller buffers (any may
  *   be NULL).
  * vip_3d_get_iters: steps taken since vip_3d_set_state, and of the last step the

@@ -519,319 +519,630 @@ __global__ void k3_scan_add(int64_t* __restrict__ out, int64_t n, const int64_t*
 }
 
 // ---- the fractional step in 3D (Sec. 2, Eqs. 12-15) ----------------------
+// The step reads its tables in slices of 32 rows (SELL-32: entry k of row r at base[r / 32]
+// + 32 k + r % 32), made from the CSR tables and point lists on the first step: a thread
+// per row then reads columns and values coalesced, where CSR rows of ~45 entries put the
+// 32 lanes of a warp on 32 lines per entry.  Rows are summed in the same order with the
+// same operations as from CSR, so the sums are the same bits.
+struct Sell3 {
+    const int64_t* base = nullptr;    // [slices + 1]
+    const int32_t* len = nullptr;     // [rows] entries of each row
+    const int32_t* col = nullptr;
+    const double* val = nullptr;
+};
+
+// Source of a step table's rows.
+enum { SRC_CSR = 0, SRC_VIP = 1, SRC_POIS = 2 };
+struct Src3 {
+    int kind, vip;           // SRC_VIP: which of the six VIPs
+    int64_t rows, N, k0;
+    Csr a, nb;               // SRC_CSR: the table; SRC_POIS: L and the Neumann rows
+    const int32_t* perm;     // row of each position (-1: none), or null: position = row
+    Asm A;
+};
+// entries [b, e) of row r, and their arrays
+__device__ __forceinline__ void src_row(const Src3& q, int64_t r, int64_t& b, int64_t& e, const int32_t*& col,
+                                        const double*& val) {
+    b = e = 0;
+    col = q.a.col;
+    val = q.a.val;
+    if (q.perm) r = q.perm[r];
+    if (r < 0 || (q.kind == SRC_CSR && r >= q.N)) return;
+    if (q.kind == SRC_CSR) {
+        b = q.a.ptr[r];
+        e = q.a.ptr[r + 1];
+    } else if (q.kind == SRC_VIP) {
+        const int32_t i = q.A.ipos[r];
+        if (i < 0) return;
+        const int64_t p = q.A.a.N + (int64_t)q.vip * q.A.a.Ni + i;
+        col = q.A.pidx;
+        val = q.A.w0 - q.A.nnz_nodes;
+        b = q.A.pptr[p];
+        e = q.A.pptr[p + 1];
+    } else if (r != q.k0) {  // row k0 holds its diagonal only, row N the equation of k0
+        const bool wall = r < q.N && q.A.ipos[r] < 0;
+        const Csr& t = wall ? q.nb : q.a;
+        const int64_t row = r == q.N ? q.k0 : r;
+        col = t.col;
+        val = t.val;
+        b = t.ptr[row];
+        e = t.ptr[row + 1];
+    }
+}
+
+__global__ void k3_sell_size(Src3 q, int64_t nsl, int32_t* __restrict__ len, int32_t* __restrict__ size) {
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // whole warps: a slice each
+    if (r >= nsl * 32) return;
+    int n = 0;
+    if (r < q.rows) {
+        int64_t b, e;
+        const int32_t* col;
+        const double* val;
+        src_row(q, r, b, e, col, val);
+        n = (int)(e - b);
+        len[r] = n;
+    }
+    const int w = __reduce_max_sync(0xffffffffu, n);
+    if ((r & 31) == 0) size[r >> 5] = w * 32;
+}
+
+__global__ void k3_sell_fill(Src3 q, const int64_t* __restrict__ base, int32_t* __restrict__ scol,
+                             double* __restrict__ sval) {
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t sl = r >> 5;
+    if (sl * 32 >= q.rows) return;
+    int64_t b = 0, e = 0;
+    const int32_t* col = nullptr;
+    const double* val = nullptr;
+    if (r < q.rows) src_row(q, r, b, e, col, val);
+    const int w = (int)((base[sl + 1] - base[sl]) >> 5);
+    for (int k = 0; k < w; ++k) {
+        const int64_t o = base[sl] + 32 * k + (r & 31);
+        const bool in = b + k < e;
+        scol[o] = in ? col[b + k] : 0;
+        sval[o] = in ? val[b + k] : 0.0;
+    }
+}
+
+// sum_k a_rk x[f][col_rk] for NF fields through one row, in entry order, one chain per
+// field.  The chain is serial and each batch of entries two dependent trips (indices,
+// gathers), so both run ahead of it: while batch k is added, batch k + 1's values and
+// gathers and batch k + 2's indices are on their way.
+template <int NF>
+__device__ __forceinline__ void row_sums(const int32_t* __restrict__ col, const double* __restrict__ val, int len,
+                                         const double* const (&x)[NF], double (&out)[NF]) {
+    constexpr int U = NF == 1 ? 8 : 4;
+    int c0[U], c1[U];
+    double a0[U], a1[U], g0[NF][U], g1[NF][U];
+    auto index = [&](int (&c)[U], int k0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) c[u] = k0 + u < len ? col[32 * (k0 + u)] : 0;
+    };
+    auto fetch = [&](const int (&c)[U], double (&a)[U], double (&g)[NF][U], int k0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool in = k0 + u < len;
+            a[u] = in ? val[32 * (k0 + u)] : 0.0;
+#pragma unroll
+            for (int f = 0; f < NF; ++f) g[f][u] = in ? x[f][c[u]] : 0.0;
+        }
+    };
+    auto add = [&](const double (&a)[U], const double (&g)[NF][U], int k0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (k0 + u < len) {
+#pragma unroll
+                for (int f = 0; f < NF; ++f) out[f] = fma(a[u], g[f][u], out[f]);
+            }
+    };
+#pragma unroll
+    for (int f = 0; f < NF; ++f) out[f] = 0.0;
+    index(c0, 0);
+    index(c1, U);
+    fetch(c0, a0, g0, 0);
+#pragma unroll 1
+    for (int k0 = 0; k0 < len; k0 += 2 * U) {
+        fetch(c1, a1, g1, k0 + U);
+        index(c0, k0 + 2 * U);
+        add(a0, g0, k0);
+        fetch(c0, a0, g0, k0 + 2 * U);
+        index(c1, k0 + 3 * U);
+        add(a1, g1, k0 + U);
+    }
+}
+template <int NF>
+__device__ __forceinline__ void sell_sums(const Sell3& t, int64_t r, const double* const (&x)[NF], double (&out)[NF]) {
+    const int64_t o = t.base[r >> 5] + (r & 31);
+    row_sums<NF>(t.col + o, t.val + o, t.len[r], x, out);
+}
+
+struct Fields3 { double* f[3]; };
+
 // Convection at every node (Sec. 4.1 item 1 in three coordinates): the products
 // of the six VIP interpolations of (u, v, w), differenced across each VIP pair
 // and divided by the pair distance.
-__global__ void k3_conv(Asm A, const double* __restrict__ u, const double* __restrict__ v,
-                        const double* __restrict__ w, double* __restrict__ Nu,
-                        double* __restrict__ Nv, double* __restrict__ Nw) {
+struct Vips3 { Sell3 t[6]; };
+__global__ void __launch_bounds__(128) k3_conv(Asm A, Vips3 T, Fields3 u, Fields3 out) {
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= A.a.N) return;
     const int32_t i = A.ipos[r];
-    if (i < 0) { Nu[r] = Nv[r] = Nw[r] = 0.0; return; }
-    double val[6][3];
-    double inv[3];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const int64_t p = A.a.N + (int64_t)k * A.a.Ni + i;
-        double su = 0.0, sv = 0.0, sw = 0.0;
-        for (int64_t s = A.pptr[p]; s < A.pptr[p + 1]; ++s) {
-            const double wt = A.w0[s - A.nnz_nodes];
-            const int32_t j = A.pidx[s];
-            su = fma(wt, u[j], su);
-            sv = fma(wt, v[j], sv);
-            sw = fma(wt, w[j], sw);
-        }
-        val[k][0] = su; val[k][1] = sv; val[k][2] = sw;
-    }
-#pragma unroll
+    if (i < 0) { out.f[0][r] = out.f[1][r] = out.f[2][r] = 0.0; return; }
+    const double* const x[3] = {u.f[0], u.f[1], u.f[2]};
+    double f[3] = {0.0, 0.0, 0.0};
+#pragma unroll 1
     for (int ax = 0; ax < 3; ++ax) {
-        double qa[3], qb[3], rho;
+        double a[3], b[3], qa[3], qb[3], rho;
         int64_t owner;
+        sell_sums<3>(T.t[2 * ax], r, x, a);
+        sell_sums<3>(T.t[2 * ax + 1], r, x, b);
         point_of(A.a, A.a.N + (int64_t)(2 * ax) * A.a.Ni + i, qa, rho, owner);
         point_of(A.a, A.a.N + (int64_t)(2 * ax + 1) * A.a.Ni + i, qb, rho, owner);
-        inv[ax] = 1.0 / fabs(qa[ax] - qb[ax]);
-    }
-    double out[3];
+        const double d = ax == 0 ? qa[0] - qb[0] : ax == 1 ? qa[1] - qb[1] : qa[2] - qb[2];
+        const double inv = 1.0 / fabs(d);
+        const double wa = ax == 0 ? a[0] : ax == 1 ? a[1] : a[2], wb = ax == 0 ? b[0] : ax == 1 ? b[1] : b[2];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        double f = 0.0;
-#pragma unroll
-        for (int ax = 0; ax < 3; ++ax)
-            f += (val[2 * ax][ax] * val[2 * ax][c] - val[2 * ax + 1][ax] * val[2 * ax + 1][c]) * inv[ax];
-        out[c] = f;
+        for (int c = 0; c < 3; ++c) f[c] += (wa * a[c] - wb * b[c]) * inv;
     }
-    Nu[r] = out[0]; Nv[r] = out[1]; Nw[r] = out[2];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) out.f[c][r] = f[c];
 }
 
-__device__ __forceinline__ double csr_row(const int64_t* __restrict__ ptr, const int32_t* __restrict__ col,
-                                          const double* __restrict__ val, int64_t r,
-                                          const double* __restrict__ x) {
-    double s = 0.0;
-    for (int64_t k = ptr[r]; k < ptr[r + 1]; ++k) s = fma(val[k], x[col[k]], s);
-    return s;
-}
-
-struct Tab3 { const int64_t* ptr; const int32_t* col; const double* val; };
-
-// Right-hand side of Eq. (12) times dt for one component at interior rows:
+// Right-hand sides of Eq. (12) times dt of the three components at interior rows:
 // (I + alpha L) u^n - dt (1.5 N^n - 0.5 N^{n-1} + G p^n); wall rows: the node's
-// boundary value.
-__global__ void k3_rhs(int64_t N, Tab3 L, Tab3 G, double alpha, double dt, const int32_t* __restrict__ ipos,
-                       const double* __restrict__ bc, const double* __restrict__ uc,
-                       const double* __restrict__ Ncur, const double* __restrict__ Nprev,
-                       const double* __restrict__ p, double* __restrict__ rhs) {
+// boundary value.  star gets the solves' initial guess u^n.
+struct Grad3 { Sell3 g[3]; };
+__global__ void __launch_bounds__(128) k3_rhs(int64_t N, Sell3 L, Grad3 G, double alpha, double dt,
+                                              const int32_t* __restrict__ ipos, Fields3 bc, Fields3 u, Fields3 Ncur,
+                                              Fields3 Nprev, const double* __restrict__ p, Fields3 rhs, Fields3 star) {
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= N) return;
-    if (ipos[r] < 0) { rhs[r] = bc[r]; return; }      // wall: the boundary value
-    const double Lu = csr_row(L.ptr, L.col, L.val, r, uc);
-    const double Gp = csr_row(G.ptr, G.col, G.val, r, p);
-    const double nab = 1.5 * Ncur[r] - 0.5 * Nprev[r];
-    rhs[r] = (uc[r] + alpha * Lu) - dt * (nab + Gp);
+    const bool inside = ipos[r] >= 0;
+    double Lu[3] = {0.0, 0.0, 0.0};
+    if (inside) {
+        const double* const x[3] = {u.f[0], u.f[1], u.f[2]};
+        sell_sums<3>(L, r, x, Lu);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const double uc = u.f[c][r];
+        star.f[c][r] = uc;
+        if (!inside) {                                // wall: the boundary value
+            rhs.f[c][r] = bc.f[c][r];
+            continue;
+        }
+        double Gp[1];
+        const double* const x[1] = {p};
+        sell_sums<1>(G.g[c], r, x, Gp);
+        const double nab = 1.5 * Ncur.f[c][r] - 0.5 * Nprev.f[c][r];
+        rhs.f[c][r] = (uc + alpha * Lu[c]) - dt * (nab + Gp[0]);
+    }
 }
 
 // Eq. (13) right-hand side, bordered: b_i = (Gx u* + Gy v* + Gz w*)_i / dt at
 // interior rows, 0 at wall rows, then b_N = b_k0 and b_k0 = 0 (k0 the first
 // interior node).
-__global__ void k3_div(int64_t N, Tab3 Gx, Tab3 Gy, Tab3 Gz, double dt, int64_t k0,
-                       const int32_t* __restrict__ ipos, const double* __restrict__ us,
-                       const double* __restrict__ vs, const double* __restrict__ ws,
-                       double* __restrict__ b) {
+__global__ void __launch_bounds__(128) k3_div(int64_t N, Grad3 G, double dt, int64_t k0,
+                                              const int32_t* __restrict__ ipos, Fields3 us, double* __restrict__ b) {
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= N) return;
     if (ipos[r] < 0) { b[r] = 0.0; return; }          // wall rows: zero normal derivative = 0
-    double d = (csr_row(Gx.ptr, Gx.col, Gx.val, r, us) + csr_row(Gy.ptr, Gy.col, Gy.val, r, vs)
-                + csr_row(Gz.ptr, Gz.col, Gz.val, r, ws)) / dt;
-    if (r == k0) { b[N] = d; b[r] = 0.0; }
-    else b[r] = d;
+    double d[3][1];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const double* const x[1] = {us.f[c]};
+        sell_sums<1>(G.g[c], r, x, d[c]);
+    }
+    const double q = (d[0][0] + d[1][0] + d[2][0]) / dt;
+    if (r == k0) { b[N] = q; b[r] = 0.0; }
+    else b[r] = q;
 }
 
 // Eqs. (14)-(15): u = u* - dt G phi at interior rows; p = p + phi - alpha L phi
 // at every node.
-__global__ void k3_project(int64_t N, Tab3 L, Tab3 Gx, Tab3 Gy, Tab3 Gz, double alpha, double dt,
-                           const int32_t* __restrict__ ipos, const double* __restrict__ phi,
-                           const double* __restrict__ us, const double* __restrict__ vs,
-                           const double* __restrict__ ws, double* __restrict__ u, double* __restrict__ v,
-                           double* __restrict__ w, double* __restrict__ p) {
+__global__ void __launch_bounds__(128) k3_project(int64_t N, Sell3 L, Grad3 G, double alpha, double dt,
+                                                  const int32_t* __restrict__ ipos, const double* __restrict__ phi,
+                                                  Fields3 us, Fields3 u, double* __restrict__ p) {
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= N) return;
-    if (ipos[r] >= 0) {
-        u[r] = us[r] - dt * csr_row(Gx.ptr, Gx.col, Gx.val, r, phi);
-        v[r] = vs[r] - dt * csr_row(Gy.ptr, Gy.col, Gy.val, r, phi);
-        w[r] = ws[r] - dt * csr_row(Gz.ptr, Gz.col, Gz.val, r, phi);
-    } else {                                          // walls keep their values
-        u[r] = us[r]; v[r] = vs[r]; w[r] = ws[r];
+    const double* const x[1] = {phi};
+    const bool inside = ipos[r] >= 0;                 // walls keep their values
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        double g[1] = {0.0};
+        if (inside) sell_sums<1>(G.g[c], r, x, g);
+        u.f[c][r] = inside ? us.f[c][r] - dt * g[0] : us.f[c][r];
     }
-    p[r] = (p[r] + phi[r]) - alpha * csr_row(L.ptr, L.col, L.val, r, phi);
+    double l[1];
+    sell_sums<1>(L, r, x, l);
+    p[r] = (p[r] + phi[r]) - alpha * l[0];
 }
 
-// The two systems of the step, applied matrix-free from L:
-//   HELM: y = x - alpha L x at interior rows, y = x at wall rows      (n = N)
+// ---- the step's linear solves ---------------------------------------------
+// The two systems, applied matrix-free from their tables:
+//   HELM: y = x - alpha L x at interior rows, y = x at wall rows      (n = N, table L)
 //   POIS: the bordered Poisson system (n = N + 1, x_N = mu): interior rows
 //         y_i = (L x)_i + mu, wall rows y_i = (-6/h_i^2) (Nb x)_i, y_k0 =
-//         (-6/h_k0^2) x_k0, y_N = (L x)_k0 + mu.
+//         (-6/h_k0^2) x_k0, y_N = (L x)_k0 + mu              (table SRC_POIS).
+// k3_bicgstab<NS> solves NS right-hand sides of one system in one cooperative launch:
+// unpreconditioned FP64 BiCGSTAB (van der Vorst 1992) to ||b - A x|| <= rtol ||b|| with the
+// oracle's rules: restart with r_hat = r when |r_hat . r| or |r_hat . v| falls below 1e-12
+// of the product of norms, and confirm convergence on the true residual.  x holds the
+// initial guess.
+//
+// The solves' tables hold their rows in an order of their own (perm): interior rows and wall
+// rows in slices apart, the wall slices spread evenly among the others.  A Neumann row is
+// about twice as long as an interior one, and in node order every lattice line ends in two,
+// so that every slice would be as wide as its wall rows.
+//
+// A block owns a run of slices.  The vectors (and the table, if it fits) stay in its shared
+// memory for the whole solve; p and s, which other blocks gather from, also go to global
+// memory.  An iteration is five phases between grid barriers, bounded by the FP64 pipe (two
+// lanes per clock and SM: 45 entries x 216 rows take 2.8 us per application at 32^3) and by
+// the barriers and reductions (about 2 us each).  Before, it was 14 launches of a
+// captured graph per iteration and a host read every few.  Step, before and now: 32^3 ABC
+// flow 3.2 -> 1.1 ms, 31^3 lid-driven cube (320 iterations) 27.8 -> 7.9 ms, 64^3 ABC flow
+// 17.7 -> 9.3 ms.  The three velocity components share the table's reads and the barriers.
 enum { OPK_HELM = 0, OPK_POIS = 1 };
-struct Op3 {
+constexpr int NV3 = 7;  // r, rhat, p, v, s, t, x
+// what a block keeps of each of its positions: the vectors, the boundary rows' scale and Pos3
+template <int NS>
+constexpr size_t pos_bytes() { return (NV3 * NS + 1) * sizeof(double) + 16; }
+enum { ROW_IN = 0, ROW_WALL = 1, ROW_PIN = 2 };
+struct Pos3 { int row, kind, len, at; };  // row (-1: none), its kind, its entries, the first one's offset
+struct Out3 {
+    int32_t it, status;
+    double relres;
+};
+template <int NS>
+struct Solve3 {
     int kind;
-    int64_t n, N, k0;
-    double alpha;
-    Tab3 L, Nb;
+    int64_t n, N, k0, nsl;
+    const int32_t* perm;     // [32 nsl] row of each position, -1: none
+    double alpha, rtol;
+    int32_t max_it;
+    Sell3 t;
     const int32_t* ipos;
     const double* h;
+    const double* rhs[NS];
+    double* x[NS];
+    double* gp[NS];          // p and s of every row
+    double* gs[NS];
+    double* work;            // pos_bytes per position, if a block's do not fit shared memory
+    int vec_smem, mat_smem;  // what the block keeps in shared memory
+    double* part;            // [2][3 NS][blocks]
+    uint32_t* bar;
+    int32_t* status;         // a failed solve stops those after it
+    Out3* out;
 };
 
-__device__ __forceinline__ double op_row(const Op3& o, int64_t r, const double* __restrict__ x) {
-    if (o.kind == OPK_HELM)
-        return o.ipos[r] >= 0 ? x[r] - o.alpha * csr_row(o.L.ptr, o.L.col, o.L.val, r, x) : x[r];
-    if (r == o.k0) return (-6.0 / (o.h[r] * o.h[r])) * x[r];
-    if (r < o.N && o.ipos[r] < 0)
-        return (-6.0 / (o.h[r] * o.h[r])) * csr_row(o.Nb.ptr, o.Nb.col, o.Nb.val, r, x);
-    const int64_t row = r == o.N ? o.k0 : r;
-    return csr_row(o.L.ptr, o.L.col, o.L.val, row, x) + x[o.N];
+__device__ __forceinline__ unsigned ld_acq3(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
 }
 
-__global__ void k3_op(Op3 o, const double* __restrict__ x, double* __restrict__ y) {
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < o.n) y[r] = op_row(o, r, x);
-}
-
-// Sum of two values over a 256-thread block, in a fixed tree; thread 0 writes them.
-__device__ __forceinline__ void block_sum2(double a, double b, double* __restrict__ out) {
-    __shared__ double s0[256], s1[256];
-    s0[threadIdx.x] = a;
-    s1[threadIdx.x] = b;
+// Grid barrier of a cooperative launch: block 0 adds 2^31 - (blocks - 1), the others 1, so the
+// counter's top bit flips when the last block arrives; every wait ends after 2 s.
+__device__ __noinline__ bool grid_sync3(uint32_t* bar, unsigned nb, int32_t* status) {
+    __shared__ int ok;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) { s0[threadIdx.x] += s0[threadIdx.x + o]; s1[threadIdx.x] += s1[threadIdx.x + o]; }
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        ok = 1;
+        const unsigned add = blockIdx.x == 0 ? 0x80000000u - (nb - 1u) : 1u;
+        unsigned old;
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(bar), "r"(add) : "memory");
+        uint64_t t0, t;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+        for (unsigned k = 1; ((ld_acq3(bar) ^ old) & 0x80000000u) == 0; ++k) {
+            if ((k & 63u) == 0) {
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+                if (t - t0 > 2000000000ull || *(volatile int32_t*)status == VIP_ERR_TIMEOUT) {
+                    atomicExch(status, VIP_ERR_TIMEOUT);
+                    ok = 0;
+                    break;
+                }
+            }
+        }
     }
-    if (threadIdx.x == 0) { out[0] = s0[0]; out[1] = s1[0]; }
-}
-
-// Deterministic dot products: fixed grid, per-thread strided sums, a fixed tree
-// in each block, then one block sums the block partials in order.
-constexpr int DOT_B = 256, DOT_T = 256;
-
-__global__ void __launch_bounds__(DOT_T) k3_dot2(int64_t n, const double* __restrict__ a,
-                                                 const double* __restrict__ b, const double* __restrict__ c,
-                                                 const double* __restrict__ d, double* __restrict__ part) {
-    __shared__ double s0[DOT_T], s1[DOT_T];
-    double x0 = 0.0, x1 = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * DOT_T + threadIdx.x; i < n; i += (int64_t)DOT_B * DOT_T) {
-        x0 = fma(a[i], b[i], x0);
-        if (c) x1 = fma(c[i], d[i], x1);
-    }
-    s0[threadIdx.x] = x0;
-    s1[threadIdx.x] = x1;
     __syncthreads();
-    for (int o = DOT_T / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) { s0[threadIdx.x] += s0[threadIdx.x + o]; s1[threadIdx.x] += s1[threadIdx.x + o]; }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) { part[2 * blockIdx.x] = s0[0]; part[2 * blockIdx.x + 1] = s1[0]; }
+    return ok != 0;
 }
 
-__global__ void __launch_bounds__(DOT_B) k3_dot_final(const double* __restrict__ part, double* __restrict__ out) {
-    __shared__ double s0[DOT_B], s1[DOT_B];
-    s0[threadIdx.x] = part[2 * threadIdx.x];
-    s1[threadIdx.x] = part[2 * threadIdx.x + 1];
-    __syncthreads();
-    for (int o = DOT_B / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) { s0[threadIdx.x] += s0[threadIdx.x + o]; s1[threadIdx.x] += s1[threadIdx.x + o]; }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) { out[0] = s0[0]; out[1] = s1[0]; }
-}
-
-// y = a x + b y' (elementwise vector updates of BiCGSTAB)
-__global__ void k3_lin2(int64_t n, double a, const double* __restrict__ x, double b,
-                        const double* __restrict__ y, double* __restrict__ out) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = a * x[i] + b * y[i];
-}
-
-// Device-resident scalars of one BiCGSTAB inner loop.  The single-thread kernels
-// below apply the same IEEE operations the host would, so the iterates do not
-// depend on where the scalars live; every vector kernel does nothing once the
-// state has left "running".
-enum { KS_RUN = 0, KS_LEAVE = 1, KS_RESTART = 2, KS_ADD_LEAVE = 3 };
-struct KS {
-    double rho, rho_old, alpha, omega, beta, rhat_norm, tol, brk;
-    double d[2];            // results of the last pair of dot products
-    int32_t it, max_it, state, pad;
+enum { S3_RESID = 0, S3_RUN = 1, S3_DONE = 2 };
+struct Sys3 {
+    double rho, rho_old, alpha, omega, beta, rhat_norm, tol, bnorm, relres;
+    int it, restarts, state, status, xadd, zero;
 };
 
-// after (r_hat . r, r . r): breakdown test, iteration count, beta
-__global__ void ks_top(KS* K) {
-    if (K->state != KS_RUN) return;
-    if (K->it >= K->max_it) { K->state = KS_LEAVE; return; }
-    const double rho = K->d[0];
-    if (fabs(rho) <= K->brk * K->rhat_norm * sqrt(K->d[1])) { K->state = KS_RESTART; return; }
-    K->rho = rho;
-    K->it += 1;
-    K->beta = (rho / K->rho_old) * (K->alpha / K->omega);
-}
-
-__global__ void ks_added(KS* K) {
-    if (K->state == KS_ADD_LEAVE) K->state = KS_LEAVE;
-}
-
-__global__ void kd_pupd(int64_t n, const KS* __restrict__ K, const double* __restrict__ r,
-                        const double* __restrict__ v, double* __restrict__ p) {
-    if (K->state != KS_RUN) return;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = r[i] + K->beta * (p[i] - K->omega * v[i]);
-}
-
-__global__ void kd_axpy_add(int64_t n, const KS* __restrict__ K, const double* __restrict__ p,
-                            double* __restrict__ x) {
-    if (K->state != KS_ADD_LEAVE) return;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) x[i] = x[i] + K->alpha * p[i];
-}
-
-// The fused kernels below write per-block partial sums of two dot products
-// (part[2 b], part[2 b + 1]); k3_final reduces them in block order and then takes
-// the iteration's scalar step.  All are launched with 256-thread blocks.
-// v = A p (mode 0: partials of r_hat . v and v . v) or t = A s (mode 1: t . t and
-// s . t); c is r_hat (mode 0) or s (mode 1).
-__global__ void __launch_bounds__(256) k3_op_dot(Op3 o, const double* __restrict__ x, double* __restrict__ y,
-                                                 const KS* __restrict__ K, const double* __restrict__ c,
-                                                 int mode, double* __restrict__ part) {
-    if (K->state != KS_RUN) return;
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double p0 = 0.0, p1 = 0.0;
-    if (r < o.n) {
-        const double yv = op_row(o, r, x);
-        y[r] = yv;
-        const double cy = c[r] * yv, yy = yv * yv;
-        p0 = mode == 0 ? cy : yy;
-        p1 = mode == 0 ? yy : cy;
+template <int NS, int NT3>
+__global__ void __launch_bounds__(NT3, 1) k3_bicgstab(Solve3<NS> a) {
+    constexpr int NW3 = NT3 / 32;
+    extern __shared__ __align__(16) double sm[];
+    constexpr int Q = 3;  // dot products of a phase, at most
+    __shared__ double red[Q * NS][NT3];
+    __shared__ double tot[Q * NS];
+    __shared__ Sys3 S[NS];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int nb = (int)gridDim.x;
+    if (*(volatile int32_t*)a.status != 0) return;  // written before this launch: the same for all blocks
+    const int64_t s0 = a.nsl * blockIdx.x / nb, s1 = a.nsl * (blockIdx.x + 1) / nb;
+    const int64_t pos0 = s0 * 32;
+    const int pitch = (int)((s1 - s0) * 32);
+    double* vec = a.vec_smem ? sm : a.work + pos0 * (pos_bytes<NS>() / 8);
+    auto V = [&](int v, int q) -> double* { return vec + (int64_t)(v * NS + q) * pitch; };
+    enum { VR, VH, VP, VV, VS, VT, VX };
+    double* scale = vec + (int64_t)NV3 * NS * pitch;
+    Pos3* pos = reinterpret_cast<Pos3*>(scale + pitch);
+    const int64_t e0 = a.t.base[s0];
+    const double* val = a.t.val + e0;
+    const int32_t* col = a.t.col + e0;
+    if (a.mat_smem) {
+        const int ne = (int)(a.t.base[s1] - e0);
+        double* sv = sm + (a.vec_smem ? (int64_t)(pos_bytes<NS>() / 8) * pitch : 0);
+        int32_t* sc = reinterpret_cast<int32_t*>(sv + ne);
+        for (int k = tid; k < ne; k += NT3) {
+            sv[k] = val[k];
+            sc[k] = col[k];
+        }
+        val = sv;
+        col = sc;
     }
-    block_sum2(p0, p1, part + 2 * blockIdx.x);
-}
-
-// s = r - alpha v; partials of s . s
-__global__ void __launch_bounds__(256) kd_s_dot(int64_t n, const KS* __restrict__ K, const double* __restrict__ r,
-                                                const double* __restrict__ v, double* __restrict__ s,
-                                                double* __restrict__ part) {
-    if (K->state != KS_RUN) return;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double p0 = 0.0;
-    if (i < n) {
-        const double sv = r[i] - K->alpha * v[i];
-        s[i] = sv;
-        p0 = sv * sv;
+    for (int i = tid; i < pitch; i += NT3) {
+        int r = __ldg(a.perm + pos0 + i);
+        if (r >= a.n) r = -1;
+        int kind = ROW_IN;
+        double sc = 1.0;
+        if (r >= 0 && r < a.N && a.ipos[r] < 0) kind = ROW_WALL;
+        if (a.kind == OPK_POIS && r == a.k0) kind = ROW_PIN;
+        if (a.kind == OPK_POIS && kind != ROW_IN) sc = -6.0 / (a.h[r] * a.h[r]);
+        const bool none = r < 0 || (a.kind == OPK_HELM ? kind == ROW_WALL : kind == ROW_PIN);
+        pos[i] = Pos3{r, kind, none ? 0 : a.t.len[pos0 + i], (int)(a.t.base[s0 + (i >> 5)] - e0) + (i & 31)};
+        scale[i] = sc;
+        if (r >= 0)
+#pragma unroll
+            for (int q = 0; q < NS; ++q) V(VX, q)[i] = a.x[q][r];
     }
-    block_sum2(p0, 0.0, part + 2 * blockIdx.x);
-}
-
-// x = x + alpha p + omega s; r = s - omega t; partials of r_hat . r and r . r
-__global__ void __launch_bounds__(256) kd_xr_dot(int64_t n, const KS* __restrict__ K, const double* __restrict__ p,
-                                                 const double* __restrict__ s, const double* __restrict__ t,
-                                                 const double* __restrict__ rhat, double* __restrict__ x,
-                                                 double* __restrict__ r, double* __restrict__ part) {
-    if (K->state != KS_RUN) return;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    double p0 = 0.0, p1 = 0.0;
-    if (i < n) {
-        x[i] = x[i] + K->alpha * p[i] + K->omega * s[i];
-        const double rv = s[i] - K->omega * t[i];
-        r[i] = rv;
-        p0 = rhat[i] * rv;
-        p1 = rv * rv;
-    }
-    block_sum2(p0, p1, part + 2 * blockIdx.x);
-}
-
-// Reduce nblk pairs of partials in block order into K->d, then the scalar step:
-//   ALPHA  (r_hat . v, v . v): breakdown test, alpha = rho / r_hat . v
-//   S      (s . s): converged on s -> x += alpha p, leave
-//   OMEGA  (t . t, s . t): omega (t = 0 -> x += alpha p, leave)
-//   END    (r_hat . r, r . r): converged or omega = 0 -> leave, else rho_old = rho
-// (the next iteration's ks_top reads r_hat . r and r . r from K->d).
-enum { FIN_ALPHA = 0, FIN_S = 1, FIN_OMEGA = 2, FIN_END = 3 };
-__global__ void __launch_bounds__(256) k3_final(const double* __restrict__ part, int nblk, KS* __restrict__ K,
-                                                int which) {
-    double a = 0.0, b = 0.0;
-    for (int k = threadIdx.x; k < nblk; k += 256) { a += part[2 * k]; b += part[2 * k + 1]; }
-    __shared__ double d[2];
-    block_sum2(a, b, d);
+    auto row_at = [&](int i) -> int { return pos[i].row; };
+    if (tid < NS) S[tid] = Sys3{};  // state S3_RESID
     __syncthreads();
-    if (threadIdx.x != 0 || K->state != KS_RUN) return;
-    K->d[0] = d[0];
-    K->d[1] = d[1];
-    if (which == FIN_ALPHA) {
-        if (fabs(d[0]) <= K->brk * K->rhat_norm * sqrt(d[1])) { K->state = KS_RESTART; return; }
-        K->alpha = K->rho / d[0];
-    } else if (which == FIN_S) {
-        if (sqrt(d[0]) <= K->tol) K->state = KS_ADD_LEAVE;
-    } else if (which == FIN_OMEGA) {
-        if (d[0] == 0.0) { K->state = KS_ADD_LEAVE; return; }
-        K->omega = d[1] / d[0];
-    } else {
-        if (sqrt(d[1]) <= K->tol || K->omega == 0.0) { K->state = KS_LEAVE; return; }
-        K->rho_old = K->rho;
+    // A applied to NS gathered vectors at position i
+    auto apply = [&](int i, const Pos3& p, const double* const (&in)[NS], double (&y)[NS]) {
+        row_sums<NS>(col + p.at, val + p.at, p.len, in, y);
+#pragma unroll
+        for (int q = 0; q < NS; ++q) {
+            if (a.kind == OPK_HELM) y[q] = p.kind == ROW_WALL ? in[q][p.row] : in[q][p.row] - a.alpha * y[q];
+            else if (p.kind == ROW_PIN) y[q] = scale[i] * in[q][p.row];
+            else y[q] = p.kind == ROW_WALL ? scale[i] * y[q] : y[q] + in[q][a.N];
+        }
+    };
+    // totals of nq quantities per system (index Q q + k): each thread's sums, 8 or 16 of them
+    // per lane of one warp, a butterfly, then the blocks' partials in block order (two
+    // alternating sets)
+    int pset = 0;
+    auto reduce = [&](const double (&d)[Q * NS], int nq) -> bool {
+#pragma unroll
+        for (int k = 0; k < Q * NS; ++k)
+            if (k % Q < nq) red[k][tid] = d[k];
+        __syncthreads();
+        double* part = a.part + (int64_t)pset * Q * NS * nb;
+        pset ^= 1;
+#pragma unroll 1
+        for (int j = warp; j < nq * NS; j += NW3) {
+            const int k = j / nq * Q + j % nq;
+            const double* p = red[k] + lane;
+            double w = 0.0;
+#pragma unroll
+            for (int t = 0; t < NT3; t += 256)
+                w += ((p[t] + p[t + 32]) + (p[t + 64] + p[t + 96])) + ((p[t + 128] + p[t + 160]) + (p[t + 192] + p[t + 224]));
+            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+            if (lane == 0) __stcg(part + (int64_t)k * nb + blockIdx.x, w);
+        }
+        if (!grid_sync3(a.bar, (unsigned)nb, a.status)) return false;
+#pragma unroll 1
+        for (int j = warp; j < nq * NS; j += NW3) {
+            const int k = j / nq * Q + j % nq;
+            double w = 0.0;
+            for (int b = lane; b < nb; b += 5 * 32) {
+                double g[5];
+#pragma unroll
+                for (int u = 0; u < 5; ++u) g[u] = b + 32 * u < nb ? __ldcg(part + (int64_t)k * nb + b + 32 * u) : 0.0;
+                w += ((g[0] + g[1]) + (g[2] + g[3])) + g[4];
+            }
+            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+            if (lane == 0) tot[k] = w;
+        }
+        __syncthreads();
+        return true;
+    };
+    static_assert(NT3 % 256 == 0, "eight values per lane at a time");
+    constexpr double BRK = 1e-12;
+    // a system's next direction, after (r_hat . r, r . r)
+    auto top = [&](Sys3& st, double rho, double rr) {
+        if (st.it >= a.max_it || fabs(rho) <= BRK * st.rhat_norm * sqrt(rr)) {
+            st.state = S3_RESID;
+            return;
+        }
+        st.rho = rho;
+        st.it += 1;
+        st.beta = (rho / st.rho_old) * (st.alpha / st.omega);
+    };
+    bool first = true, alive = true;
+    while (alive) {
+        if (__syncthreads_or(tid < NS && S[tid].state == S3_RESID)) {
+            if (!first) {  // the iterate to global memory, where its neighbours gather it
+                for (int i = tid; i < pitch; i += NT3) {
+                    const int r = row_at(i);
+                    if (r < 0) continue;
+#pragma unroll
+                    for (int q = 0; q < NS; ++q)
+                        if (S[q].state == S3_RESID) {
+                            double xv = V(VX, q)[i];
+                            if (S[q].xadd) V(VX, q)[i] = xv = xv + S[q].alpha * V(VP, q)[i];
+                            a.x[q][r] = xv;
+                        }
+                }
+                if (!grid_sync3(a.bar, (unsigned)nb, a.status)) return;
+            }
+            double d[Q * NS] = {};
+            for (int i = tid; i < pitch; i += NT3) {
+                const Pos3 ps = pos[i];
+                const int r = ps.row;
+                if (r < 0) continue;
+                const double* in[NS];
+                double y[NS];
+#pragma unroll
+                for (int q = 0; q < NS; ++q) in[q] = a.x[q];
+                apply(i, ps, in, y);
+#pragma unroll
+                for (int q = 0; q < NS; ++q)
+                    if (S[q].state == S3_RESID) {
+                        const double b = a.rhs[q][r], res = b - y[q];
+                        V(VR, q)[i] = res;
+                        V(VH, q)[i] = res;
+                        V(VP, q)[i] = 0.0;
+                        V(VV, q)[i] = 0.0;
+                        d[Q * q] = fma(res, res, d[Q * q]);
+                        d[Q * q + 1] = fma(b, b, d[Q * q + 1]);
+                    }
+            }
+            if (!reduce(d, 2)) return;
+            if (tid < NS && S[tid].state == S3_RESID) {
+                Sys3& st = S[tid];
+                const double rr = tot[Q * tid];
+                st.xadd = 0;
+                if (first) {
+                    st.bnorm = sqrt(tot[Q * tid + 1]);
+                    st.tol = a.rtol * st.bnorm;
+                }
+                const double rn = sqrt(rr);
+                if (!isfinite(st.bnorm)) {
+                    st.state = S3_DONE;
+                    st.status = VIP_ERR_NONFINITE;
+                } else if (st.bnorm == 0.0) {  // x = 0 solves A x = 0
+                    st.state = S3_DONE;
+                    st.zero = 1;
+                } else if (!isfinite(rr)) {
+                    st.state = S3_DONE;
+                    st.status = VIP_ERR_NONFINITE;
+                } else if (rn <= st.tol || st.it >= a.max_it) {
+                    st.state = S3_DONE;
+                    st.relres = rn / st.bnorm;
+                    if (rn > st.tol && st.relres > a.rtol) st.status = VIP_ERR_NOT_CONVERGED;
+                } else if (++st.restarts > 1000) {
+                    st.state = S3_DONE;
+                    st.status = VIP_ERR_BREAKDOWN;
+                } else {
+                    st.state = S3_RUN;
+                    st.rho_old = st.alpha = st.omega = 1.0;
+                    st.rhat_norm = rn;
+                    top(st, rr, rr);
+                }
+            }
+            first = false;
+            if (__syncthreads_or(tid < NS && S[tid].state == S3_RESID)) continue;
+        }
+        if (!__syncthreads_or(tid < NS && S[tid].state == S3_RUN)) break;
+        // v = A p, p = r + beta (p - omega v) (half 0), or t = A s, s = r - alpha v (half 1),
+        // with their dot products; s . s is tested with those of t (a converged s wastes
+        // the last application, and every iteration saves a reduction)
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+            double d[Q * NS] = {};
+            for (int i = tid; i < pitch; i += NT3) {
+                const int r = row_at(i);
+                if (r < 0) continue;
+#pragma unroll
+                for (int q = 0; q < NS; ++q)
+                    if (S[q].state == S3_RUN) {
+                        const double rv = V(VR, q)[i], vv = V(VV, q)[i];
+                        if (!half) {
+                            const double pv = rv + S[q].beta * (V(VP, q)[i] - S[q].omega * vv);
+                            V(VP, q)[i] = pv;
+                            a.gp[q][r] = pv;
+                        } else {
+                            const double sv = rv - S[q].alpha * vv;
+                            V(VS, q)[i] = sv;
+                            a.gs[q][r] = sv;
+                        }
+                    }
+            }
+            if (!grid_sync3(a.bar, (unsigned)nb, a.status)) return;
+            for (int i = tid; i < pitch; i += NT3) {
+                const Pos3 ps = pos[i];
+                const int r = ps.row;
+                if (r < 0) continue;
+                const double* in[NS];
+                double y[NS];
+#pragma unroll
+                for (int q = 0; q < NS; ++q) in[q] = half ? a.gs[q] : a.gp[q];
+                apply(i, ps, in, y);
+#pragma unroll
+                for (int q = 0; q < NS; ++q)
+                    if (S[q].state == S3_RUN) {
+                        V(half ? VT : VV, q)[i] = y[q];
+                        const double c = V(half ? VS : VH, q)[i];
+                        d[Q * q] = fma(c, y[q], d[Q * q]);              // r_hat . v or s . t
+                        d[Q * q + 1] = fma(y[q], y[q], d[Q * q + 1]);   // v . v or t . t
+                        if (half) d[Q * q + 2] = fma(c, c, d[Q * q + 2]);
+                    }
+            }
+            if (!reduce(d, 2 + half)) return;
+            if (tid < NS && S[tid].state == S3_RUN) {
+                Sys3& st = S[tid];
+                const double cy = tot[Q * tid], yy = tot[Q * tid + 1];
+                if (!isfinite(cy) || !isfinite(yy)) {
+                    st.state = S3_DONE;
+                    st.status = VIP_ERR_NONFINITE;
+                } else if (!half) {
+                    if (fabs(cy) <= BRK * st.rhat_norm * sqrt(yy)) st.state = S3_RESID;
+                    else st.alpha = st.rho / cy;
+                } else if (sqrt(tot[Q * tid + 2]) <= st.tol || yy == 0.0) {
+                    st.xadd = 1;  // x += alpha p
+                    st.state = S3_RESID;
+                } else {
+                    st.omega = cy / yy;
+                }
+            }
+            __syncthreads();
+        }
+        // x += alpha p + omega s;  r = s - omega t
+        double d[Q * NS] = {};
+        for (int i = tid; i < pitch; i += NT3) {
+            if (row_at(i) < 0) continue;
+#pragma unroll
+            for (int q = 0; q < NS; ++q)
+                if (S[q].state == S3_RUN) {
+                    const double sv = V(VS, q)[i];
+                    V(VX, q)[i] = V(VX, q)[i] + S[q].alpha * V(VP, q)[i] + S[q].omega * sv;
+                    const double rv = sv - S[q].omega * V(VT, q)[i];
+                    V(VR, q)[i] = rv;
+                    d[Q * q] = fma(V(VH, q)[i], rv, d[Q * q]);
+                    d[Q * q + 1] = fma(rv, rv, d[Q * q + 1]);
+                }
+        }
+        if (!reduce(d, 2)) return;
+        if (tid < NS && S[tid].state == S3_RUN) {
+            Sys3& st = S[tid];
+            const double rho = tot[Q * tid], rr = tot[Q * tid + 1];
+            if (!isfinite(rho) || !isfinite(rr)) {
+                st.state = S3_DONE;
+                st.status = VIP_ERR_NONFINITE;
+            } else if (sqrt(rr) <= st.tol || st.omega == 0.0) {
+                st.state = S3_RESID;
+            } else {
+                st.rho_old = st.rho;
+                top(st, rho, rr);
+            }
+        }
+        __syncthreads();
+    }
+    for (int i = tid; i < pitch; i += NT3)
+#pragma unroll
+        for (int q = 0; q < NS; ++q)
+            if (S[q].zero && row_at(i) >= 0) a.x[q][row_at(i)] = 0.0;
+    if (blockIdx.x == 0 && tid < NS) {
+        a.out[tid] = Out3{S[tid].it, S[tid].status, S[tid].relres};
+        if (S[tid].status) atomicCAS(a.status, 0, S[tid].status);
     }
 }
 
@@ -844,6 +1155,7 @@ inline unsigned blocks_for(int64_t n, int t) { return (unsigned)std::max<int64_t
 // ---------------------------------------------------------------------------
 struct vip_3d {
     int device = 0;
+    int sms = 0, smem = 0;            // multiprocessors; dynamic shared memory of a solve block
     cudaStream_t stream = nullptr;
     std::string err;
     int weight = VIP_W_CUBIC_SPLINE;
@@ -878,15 +1190,18 @@ struct vip_3d {
     double *p = nullptr, *phi = nullptr;          // phi: N + 1 (mu last)
     int64_t k0 = -1;                              // first interior node
     bool other_kinds = false;                     // SLIP or OUTLET nodes present
-    double* kv[8] = {};                           // Krylov vectors, N + 1 each
-    double *dpart = nullptr, *dres = nullptr;     // dot partials and results
-    void* ks = nullptr;                           // device BiCGSTAB scalars (KS)
-    // one BiCGSTAB inner iteration as a CUDA graph per (system, solution vector),
-    // captured on a private stream and replayed on `stream`; dropped whenever a
-    // table, the flow parameters or the step's buffers change
-    struct IterGraph { int kind; const double* x; cudaGraphExec_t exec; };
-    std::vector<IterGraph> graphs;
-    cudaStream_t cap = nullptr;
+    double* rhs[3] = {nullptr, nullptr, nullptr}; // right-hand sides, N + 1 each (Poisson: the first)
+    double* gather[2][3] = {};                    // p and s of the solves, N + 1 each
+    double* work = nullptr;                       // Krylov vectors of blocks that exceed shared memory
+    double* dpart = nullptr;                      // dot-product partials
+    Out3* dout = nullptr;                         // [4] results of a step's solves
+    uint32_t* dbar = nullptr;                     // [2] barrier word, status
+    // the step's tables in slices, made on the first step after a build
+    bool sliced = false;
+    Sell3 sl_lap, sl_helm, sl_pois, sl_grad[3], sl_vip[6];
+    int32_t* perm = nullptr;                      // the solves' row order (see Solve3)
+    int64_t nsl = 0;                              // its slices
+    int64_t ent_helm = 0, ent_pois = 0;           // most entries of a block's slices
     int64_t steps = 0;
     int32_t last_helm = 0, last_poisson = 0;
     double last_poisson_res = 0.0;
@@ -923,15 +1238,10 @@ void free_all(std::vector<void*>& v) {
     v.clear();
 }
 
-void drop_graphs(vip_3d* b) {
-    for (auto& g : b->graphs) cudaGraphExecDestroy(g.exec);
-    b->graphs.clear();
-}
-
 void reset_build(vip_3d* b) {
-    drop_graphs(b);
     free_all(b->build_bufs);
-    b->built = false;
+    b->built = b->sliced = false;
+    b->work = nullptr;
     for (int i = 0; i < VIP3_OP_COUNT; ++i) { b->tab[i] = Csr{}; b->have[i] = false; }
     b->pptr = nullptr; b->pidx = nullptr; b->wnode = nullptr; b->w0 = nullptr;
     b->P = b->nnz_all = b->nnz_nodes = 0;
@@ -1016,126 +1326,148 @@ vip_status assemble(vip_3d* b, int op) {
     return VIP_OK;
 }
 
-Tab3 tab3(const vip_3d* b, int op) {
-    return Tab3{b->tab[op].ptr, b->tab[op].col, b->tab[op].val};
-}
-
-// Two dot products (the second optional) of device vectors, read back to the host.
-vip_status dots(vip_3d* b, int64_t n, const double* a1, const double* b1, const double* a2,
-                const double* b2, double out[2]) {
-    k3_dot2<<<DOT_B, DOT_T, 0, b->stream>>>(n, a1, b1, a2, b2, b->dpart);
-    k3_dot_final<<<1, DOT_B, 0, b->stream>>>(b->dpart, b->dres);
-    V3_CUDA(cudaGetLastError());
-    V3_CUDA(cudaMemcpyAsync(out, b->dres, 2 * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
-    V3_CUDA(cudaStreamSynchronize(b->stream));
-    return VIP_OK;
-}
-
 #define V3_TRY(call)                          \
     do {                                      \
         vip_status s_ = (call);               \
         if (s_ != VIP_OK) return s_;          \
     } while (0)
 
-// Unpreconditioned BiCGSTAB (van der Vorst 1992) on o to ||rhs - A x|| <= rtol ||rhs||,
-// with the oracle's rules: restart with r_hat = r when |r_hat . r| or |r_hat . v|
-// falls below 1e-12 of the product of norms, and confirm convergence on the true
-// residual.  x holds the initial guess.
-vip_status krylov(vip_3d* b, const Op3& o, const double* rhs, double* x, int32_t* iters, double* relres) {
-    const int64_t n = o.n;
-    double *r = b->kv[0], *rhat = b->kv[1], *pp = b->kv[2], *v = b->kv[3], *sv = b->kv[4],
-           *t = b->kv[5], *y = b->kv[6];
-    KS* K = static_cast<KS*>(b->ks);
-    const unsigned g = blocks_for(n, 256);
-    cudaStream_t st = b->stream;
-    auto apply = [&](const double* in, double* out) { k3_op<<<g, 256, 0, st>>>(o, in, out); };
-    // one inner iteration, enqueued on stream q (captured once into a graph): 14
-    // kernels, the dot products fused into the operator and vector kernels
-    const int nblk = (int)g;
-    double* part = b->dpart;
-    auto iteration = [&](cudaStream_t q) {
-        ks_top<<<1, 1, 0, q>>>(K);
-        kd_pupd<<<g, 256, 0, q>>>(n, K, r, v, pp);
-        k3_op_dot<<<g, 256, 0, q>>>(o, pp, v, K, rhat, 0, part);
-        k3_final<<<1, 256, 0, q>>>(part, nblk, K, FIN_ALPHA);
-        kd_s_dot<<<g, 256, 0, q>>>(n, K, r, v, sv, part);
-        k3_final<<<1, 256, 0, q>>>(part, nblk, K, FIN_S);
-        kd_axpy_add<<<g, 256, 0, q>>>(n, K, pp, x);
-        ks_added<<<1, 1, 0, q>>>(K);
-        k3_op_dot<<<g, 256, 0, q>>>(o, sv, t, K, sv, 1, part);
-        k3_final<<<1, 256, 0, q>>>(part, nblk, K, FIN_OMEGA);
-        kd_axpy_add<<<g, 256, 0, q>>>(n, K, pp, x);
-        ks_added<<<1, 1, 0, q>>>(K);
-        kd_xr_dot<<<g, 256, 0, q>>>(n, K, pp, sv, t, rhat, x, r, part);
-        k3_final<<<1, 256, 0, q>>>(part, nblk, K, FIN_END);
-    };
-    cudaGraphExec_t exec = nullptr;
-    for (const auto& gr : b->graphs)
-        if (gr.kind == o.kind && gr.x == x) exec = gr.exec;
-    if (!exec) {
-        if (!b->cap) V3_CUDA(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
-        cudaGraph_t graph = nullptr;
-        V3_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
-        iteration(b->cap);
-        cudaError_t ce = cudaStreamEndCapture(b->cap, &graph);
-        if (ce == cudaSuccess) ce = cudaGraphInstantiate(&exec, graph, 0);
-        if (graph) cudaGraphDestroy(graph);
-        V3_CUDA(ce);
-        b->graphs.push_back({o.kind, x, exec});
+// blocks of a solve over n rows: one per SM, at least a slice each
+int solve_blocks(const vip_3d* b) { return (int)std::max<int64_t>(1, std::min<int64_t>(b->sms, b->nsl)); }
+
+// A step table in slices; *most gets the largest entry count of a solve block's slices.
+vip_status slice_table(vip_3d* b, const Src3& q, Sell3& t, int64_t* most) {
+    const int64_t nsl = (q.rows + 31) / 32;
+    int32_t *len = nullptr, *size = nullptr, *col = nullptr;
+    int64_t *base = nullptr, nent = 0;
+    double* val = nullptr;
+    V3_CUDA(alloc(b->build_bufs, &len, q.rows));
+    V3_CUDA(alloc(b->build_bufs, &base, nsl + 1));
+    std::vector<void*> tmp;
+    cudaError_t e = alloc(tmp, &size, nsl);
+    if (e != cudaSuccess) { free_all(tmp); V3_CUDA(e); }
+    k3_sell_size<<<blocks_for(nsl * 32, 256), 256, 0, b->stream>>>(q, nsl, len, size);
+    vip_status st = scan_counts(b, size, nsl, base, &nent);
+    free_all(tmp);
+    if (st != VIP_OK) return st;
+    V3_CUDA(alloc(b->build_bufs, &col, nent));
+    V3_CUDA(alloc(b->build_bufs, &val, nent));
+    k3_sell_fill<<<blocks_for(nsl * 32, 256), 256, 0, b->stream>>>(q, base, col, val);
+    V3_CUDA(cudaGetLastError());
+    t.base = base; t.len = len; t.col = col; t.val = val;
+    if (most) {
+        std::vector<int64_t> hb(nsl + 1);
+        V3_CUDA(cudaMemcpyAsync(hb.data(), base, (nsl + 1) * 8, cudaMemcpyDeviceToHost, b->stream));
+        V3_CUDA(cudaStreamSynchronize(b->stream));
+        const int nb = solve_blocks(b);
+        *most = 0;
+        for (int k = 0; k < nb; ++k) *most = std::max(*most, hb[nsl * (k + 1) / nb] - hb[nsl * k / nb]);
     }
-    double d[2];
-    V3_TRY(dots(b, n, rhs, rhs, nullptr, nullptr, d));
-    const double bnorm = std::sqrt(d[0]);
-    *iters = 0;
-    *relres = 0.0;
-    if (!std::isfinite(bnorm)) return fail(b, VIP_ERR_NONFINITE, "non-finite right-hand side");
-    if (bnorm == 0.0) {
-        V3_CUDA(cudaMemsetAsync(x, 0, n * sizeof(double), st));
-        return VIP_OK;
-    }
-    const double tol = b->rtol * bnorm;
-    // inner iterations launched between host reads: 1, 2, 4, ... 16, so that a solve
-    // of a few iterations (the Helmholtz ones) launches few that do nothing
-    constexpr int CHUNK_MAX = 16;
-    int32_t it = 0, restarts = 0;
-    while (it < b->max_iters) {
-        apply(x, y);
-        k3_lin2<<<g, 256, 0, st>>>(n, 1.0, rhs, -1.0, y, r);
-        V3_TRY(dots(b, n, r, r, nullptr, nullptr, d));
-        if (!std::isfinite(d[0])) return fail(b, VIP_ERR_NONFINITE, "non-finite residual");
-        if (std::sqrt(d[0]) <= tol) break;
-        if (++restarts > 1000) return fail(b, VIP_ERR_BREAKDOWN, "BiCGSTAB: no progress after 1000 restarts");
-        V3_CUDA(cudaMemcpyAsync(rhat, r, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
-        KS h{};
-        h.rho_old = h.alpha = h.omega = 1.0;
-        h.rhat_norm = std::sqrt(d[0]);
-        h.tol = tol;
-        h.brk = 1e-12;
-        h.it = it;
-        h.max_it = b->max_iters;
-        h.state = KS_RUN;
-        h.d[0] = h.d[1] = d[0];       // r_hat . r and r . r, with r_hat = r
-        V3_CUDA(cudaMemcpyAsync(K, &h, sizeof(KS), cudaMemcpyHostToDevice, st));
-        V3_CUDA(cudaMemsetAsync(v, 0, n * sizeof(double), st));
-        V3_CUDA(cudaMemsetAsync(pp, 0, n * sizeof(double), st));
-        for (int chunk = 1;; chunk = std::min(2 * chunk, CHUNK_MAX)) {
-            for (int c = 0; c < chunk; ++c) V3_CUDA(cudaGraphLaunch(exec, st));
-            V3_CUDA(cudaGetLastError());
-            V3_CUDA(cudaMemcpyAsync(&h, K, sizeof(KS), cudaMemcpyDeviceToHost, st));
-            V3_CUDA(cudaStreamSynchronize(st));
-            it = h.it;
-            if (!std::isfinite(h.d[0])) return fail(b, VIP_ERR_NONFINITE, "non-finite residual");
-            if (h.state != KS_RUN) break;
-        }
-    }
-    apply(x, y);
-    k3_lin2<<<g, 256, 0, st>>>(n, 1.0, rhs, -1.0, y, r);
-    V3_TRY(dots(b, n, r, r, nullptr, nullptr, d));
-    *iters = it;
-    *relres = std::sqrt(d[0]) / bnorm;
-    if (!std::isfinite(*relres)) return fail(b, VIP_ERR_NONFINITE, "non-finite solution");
-    if (*relres > b->rtol) return fail(b, VIP_ERR_NOT_CONVERGED, "BiCGSTAB hit its iteration limit");
     return VIP_OK;
+}
+
+vip_status slice_tables(vip_3d* b) {
+    if (b->sliced) return VIP_OK;
+    const int need[5] = {VIP3_OP_LAPLACE, VIP3_OP_GX, VIP3_OP_GY, VIP3_OP_GZ, VIP3_OP_NEUMANN};
+    for (int op : need) V3_TRY(assemble(b, op));
+    Src3 q{};
+    q.A = asm_view(b);
+    q.N = b->N;
+    q.k0 = b->k0;
+    q.kind = SRC_CSR;
+    q.rows = b->N;
+    q.a = b->tab[VIP3_OP_LAPLACE];
+    V3_TRY(slice_table(b, q, b->sl_lap, nullptr));
+    for (int c = 0; c < 3; ++c) {
+        q.a = b->tab[VIP3_OP_GX + c];
+        V3_TRY(slice_table(b, q, b->sl_grad[c], nullptr));
+    }
+    q.kind = SRC_VIP;
+    for (int k = 0; k < 6; ++k) {
+        q.vip = k;
+        V3_TRY(slice_table(b, q, b->sl_vip[k], nullptr));
+    }
+    // the solves' row order: interior rows (and the border row N), wall rows, each padded to
+    // whole slices; wall slice j of nw goes after (j + 1) / nw of the others
+    std::vector<int32_t> ip(b->N), in, wall, perm;
+    V3_CUDA(cudaMemcpyAsync(ip.data(), b->ipos, b->N * 4, cudaMemcpyDeviceToHost, b->stream));
+    V3_CUDA(cudaStreamSynchronize(b->stream));
+    for (int64_t r = 0; r < b->N; ++r) (ip[r] >= 0 ? in : wall).push_back((int32_t)r);
+    in.push_back((int32_t)b->N);
+    for (auto* v : {&in, &wall}) v->resize((v->size() + 31) / 32 * 32, -1);
+    const int64_t ni = (int64_t)in.size() / 32, nw = (int64_t)wall.size() / 32;
+    b->nsl = ni + nw;
+    for (int64_t k = 0, i = 0, j = 0; k < b->nsl; ++k) {
+        const bool w = (k + 1) * nw / b->nsl > j;
+        const int32_t* src = w ? wall.data() + 32 * j++ : in.data() + 32 * i++;
+        perm.insert(perm.end(), src, src + 32);
+    }
+    V3_CUDA(alloc(b->build_bufs, &b->perm, perm.size()));
+    V3_CUDA(cudaMemcpyAsync(b->perm, perm.data(), perm.size() * 4, cudaMemcpyHostToDevice, b->stream));
+    V3_CUDA(cudaStreamSynchronize(b->stream));
+    q.perm = b->perm;
+    q.rows = 32 * b->nsl;
+    q.kind = SRC_CSR;
+    q.a = b->tab[VIP3_OP_LAPLACE];
+    V3_TRY(slice_table(b, q, b->sl_helm, &b->ent_helm));
+    q.kind = SRC_POIS;
+    q.nb = b->tab[VIP3_OP_NEUMANN];
+    V3_TRY(slice_table(b, q, b->sl_pois, &b->ent_pois));
+    b->sliced = true;
+    return VIP_OK;
+}
+
+// Enqueue the solve of NS right-hand sides; results in dout[slot ..).
+template <int NS, int NT3>
+vip_status solve_with(vip_3d* b, int kind, double* const* x, int slot) {
+    const int nb = solve_blocks(b);
+    Solve3<NS> a{};
+    a.kind = kind;
+    a.n = kind == OPK_HELM ? b->N : b->N + 1;
+    a.nsl = b->nsl;
+    a.perm = b->perm;
+    a.N = b->N; a.k0 = b->k0;
+    a.alpha = b->dt / (2.0 * b->Re);
+    a.rtol = b->rtol;
+    a.max_it = b->max_iters;
+    a.t = kind == OPK_HELM ? b->sl_helm : b->sl_pois;
+    a.ipos = b->ipos;
+    a.h = b->h;
+    for (int q = 0; q < NS; ++q) {
+        a.rhs[q] = b->rhs[q];
+        a.x[q] = x[q];
+        a.gp[q] = b->gather[0][q];
+        a.gs[q] = b->gather[1][q];
+    }
+    a.part = b->dpart;
+    a.bar = b->dbar;
+    a.status = reinterpret_cast<int32_t*>(b->dbar + 1);
+    a.out = b->dout + slot;
+    // shared memory: the vectors of the block's rows first, then its part of the table
+    const size_t most = (size_t)b->smem;
+    const size_t vb = pos_bytes<NS>() * ((b->nsl + nb - 1) / nb) * 32;
+    const size_t mb = (size_t)(kind == OPK_HELM ? b->ent_helm : b->ent_pois) * 12;
+    size_t dyn = 0;
+    if (vb <= most) { a.vec_smem = 1; dyn = vb; }
+    if (dyn + mb <= most) { a.mat_smem = 1; dyn += mb; }
+    if (!a.vec_smem) {
+        if (!b->work) V3_CUDA(alloc(b->build_bufs, &b->work, pos_bytes<3>() / 8 * 32 * b->nsl));
+        a.work = b->work;
+    }
+    V3_CUDA(cudaFuncSetAttribute(k3_bicgstab<NS, NT3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    V3_CUDA(cudaMemsetAsync(b->dbar, 0, sizeof(uint32_t), b->stream));
+    void* args[] = {&a};
+    V3_CUDA(cudaLaunchCooperativeKernel((const void*)k3_bicgstab<NS, NT3>, dim3(nb), dim3(NT3), args, dyn, b->stream));
+    return VIP_OK;
+}
+
+// 256 threads while a warp holds at most two slices (fewer to synchronise and reduce over);
+// 512 beyond, where the table streams from L2 or memory and more warps keep more of it in
+// flight (884,736 nodes: 60.6 -> 38.9 ms per step).
+template <int NS>
+vip_status solve(vip_3d* b, int kind, double* const* x, int slot) {
+    return b->nsl <= (int64_t)16 * solve_blocks(b) ? solve_with<NS, 256>(b, kind, x, slot)
+                                                   : solve_with<NS, 512>(b, kind, x, slot);
 }
 
 // One fractional step (Eqs. 12-15) on a built node set of interior and wall nodes.
@@ -1144,44 +1476,42 @@ vip_status step_once(vip_3d* b) {
     const unsigned g = blocks_for(N, 128);
     cudaStream_t st = b->stream;
     const double alpha = b->dt / (2.0 * b->Re), dt = b->dt;
-    const Tab3 L = tab3(b, VIP3_OP_LAPLACE);
-    const Tab3 Nb = b->Nb ? tab3(b, VIP3_OP_NEUMANN) : Tab3{nullptr, nullptr, nullptr};
-    const Tab3 G[3] = {tab3(b, VIP3_OP_GX), tab3(b, VIP3_OP_GY), tab3(b, VIP3_OP_GZ)};
-    k3_conv<<<g, 128, 0, st>>>(asm_view(b), b->vel[0], b->vel[1], b->vel[2], b->Ncur[0], b->Ncur[1],
-                               b->Ncur[2]);
+    auto fields = [](double* const* f) { return Fields3{{f[0], f[1], f[2]}}; };
+    const Grad3 G{{b->sl_grad[0], b->sl_grad[1], b->sl_grad[2]}};
+    Vips3 T;
+    for (int k = 0; k < 6; ++k) T.t[k] = b->sl_vip[k];
+    k3_conv<<<g, 128, 0, st>>>(asm_view(b), T, fields(b->vel), fields(b->Ncur));
     V3_CUDA(cudaGetLastError());
     if (!b->have_prev)
         for (int c = 0; c < 3; ++c)
             V3_CUDA(cudaMemcpyAsync(b->Nprev[c], b->Ncur[c], N * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    double* rhs = b->kv[7];
-    int32_t helm = 0;
-    for (int c = 0; c < 3; ++c) {
-        k3_rhs<<<g, 128, 0, st>>>(N, L, G[c], alpha, dt, b->ipos, b->bc[c], b->vel[c], b->Ncur[c],
-                                  b->Nprev[c], b->p, rhs);
-        V3_CUDA(cudaGetLastError());
-        V3_CUDA(cudaMemcpyAsync(b->star[c], b->vel[c], N * sizeof(double), cudaMemcpyDeviceToDevice, st));
-        const Op3 oh{OPK_HELM, N, N, b->k0, alpha, L, Nb, b->ipos, b->h};
-        int32_t it = 0;
-        double res = 0.0;
-        V3_TRY(krylov(b, oh, rhs, b->star[c], &it, &res));
-        helm += it;
-    }
+    k3_rhs<<<g, 128, 0, st>>>(N, b->sl_lap, G, alpha, dt, b->ipos, fields(b->bc), fields(b->vel), fields(b->Ncur),
+                              fields(b->Nprev), b->p, fields(b->rhs), fields(b->star));
+    V3_CUDA(cudaGetLastError());
+    V3_CUDA(cudaMemsetAsync(b->dbar, 0, 2 * sizeof(uint32_t), st));
+    V3_TRY(solve<3>(b, OPK_HELM, b->star, 0));
     for (int c = 0; c < 3; ++c) std::swap(b->Ncur[c], b->Nprev[c]);
     b->have_prev = true;
-    k3_div<<<g, 128, 0, st>>>(N, G[0], G[1], G[2], dt, b->k0, b->ipos, b->star[0], b->star[1], b->star[2],
-                              rhs);
+    k3_div<<<g, 128, 0, st>>>(N, G, dt, b->k0, b->ipos, fields(b->star), b->rhs[0]);
     V3_CUDA(cudaGetLastError());
-    const Op3 op{OPK_POIS, N + 1, N, b->k0, alpha, L, Nb, b->ipos, b->h};
-    int32_t itp = 0;
-    double resp = 0.0;
-    V3_TRY(krylov(b, op, rhs, b->phi, &itp, &resp));
-    k3_project<<<g, 128, 0, st>>>(N, L, G[0], G[1], G[2], alpha, dt, b->ipos, b->phi, b->star[0],
-                                  b->star[1], b->star[2], b->vel[0], b->vel[1], b->vel[2], b->p);
+    V3_TRY(solve<1>(b, OPK_POIS, &b->phi, 3));
+    k3_project<<<g, 128, 0, st>>>(N, b->sl_lap, G, alpha, dt, b->ipos, b->phi, fields(b->star), fields(b->vel), b->p);
     V3_CUDA(cudaGetLastError());
+    Out3 out[4] = {};
+    uint32_t word[2] = {0, 0};
+    V3_CUDA(cudaMemcpyAsync(out, b->dout, sizeof(out), cudaMemcpyDeviceToHost, st));
+    V3_CUDA(cudaMemcpyAsync(word, b->dbar, sizeof(word), cudaMemcpyDeviceToHost, st));
     V3_CUDA(cudaStreamSynchronize(st));
-    b->last_helm = helm;
-    b->last_poisson = itp;
-    b->last_poisson_res = resp;
+    switch ((int32_t)word[1]) {
+        case VIP_OK: break;
+        case VIP_ERR_NONFINITE: return fail(b, VIP_ERR_NONFINITE, "non-finite right-hand side, residual or solution");
+        case VIP_ERR_BREAKDOWN: return fail(b, VIP_ERR_BREAKDOWN, "BiCGSTAB: no progress after 1000 restarts");
+        case VIP_ERR_NOT_CONVERGED: return fail(b, VIP_ERR_NOT_CONVERGED, "BiCGSTAB hit its iteration limit");
+        default: return fail(b, (vip_status)word[1], "a solve's grid barrier timed out");
+    }
+    b->last_helm = out[0].it + out[1].it + out[2].it;
+    b->last_poisson = out[3].it;
+    b->last_poisson_res = out[3].relres;
     ++b->steps;
     return VIP_OK;
 }
@@ -1210,6 +1540,18 @@ vip_status vip_3d_create(vip_3d** out, int device, void* cuda_stream) {
     if (!b) return VIP_ERR_OOM;
     b->device = device;
     b->stream = static_cast<cudaStream_t>(cuda_stream);
+    // shared memory a block may have, less the solve kernel's own (its static arrays)
+    int optin = 0;
+    cudaFuncAttributes fa{};
+    DeviceScope ds(device);
+    if (!ds.ok || cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
+        cudaFuncGetAttributes(&fa, k3_bicgstab<3, 512>) != cudaSuccess) {
+        (void)cudaGetLastError();
+        delete b;
+        return VIP_ERR_CUDA;
+    }
+    b->smem = std::max(0, optin - (int)fa.sharedSizeBytes - 1024);
     *out = b;
     return VIP_OK;
 }
@@ -1217,8 +1559,6 @@ vip_status vip_3d_create(vip_3d** out, int device, void* cuda_stream) {
 void vip_3d_destroy(vip_3d* b) {
     if (!b) return;
     DeviceScope ds(b->device);
-    drop_graphs(b);
-    if (b->cap) cudaStreamDestroy(b->cap);
     free_all(b->build_bufs);
     free_all(b->node_bufs);
     free_all(b->state_bufs);
@@ -1287,9 +1627,10 @@ vip_status vip_3d_set_nodes(vip_3d* b, int64_t n, const double* x, const double*
     free_all(b->node_bufs);
     free_all(b->state_bufs);
     for (int c = 0; c < 3; ++c) b->vel[c] = b->star[c] = b->Ncur[c] = b->Nprev[c] = b->bc[c] = nullptr;
-    for (double*& q : b->kv) q = nullptr;
-    b->p = b->phi = b->dpart = b->dres = nullptr;
-    b->ks = nullptr;
+    for (int c = 0; c < 3; ++c) b->rhs[c] = b->gather[0][c] = b->gather[1][c] = nullptr;
+    b->p = b->phi = b->dpart = nullptr;
+    b->dout = nullptr;
+    b->dbar = nullptr;
     b->state = b->have_prev = false;
     b->steps = 0;
     b->N = 0;
@@ -1483,7 +1824,6 @@ vip_status vip_3d_set_flow(vip_3d* b, double Re, double dt, double rtol, int32_t
         return fail(b, VIP_ERR_ARG, "Re and dt must be finite and > 0");
     if (!(rtol > 0.0 && rtol < 1.0)) return fail(b, VIP_ERR_ARG, "rtol must lie in (0, 1)");
     if (max_iters < 1) return fail(b, VIP_ERR_ARG, "max_iters must be >= 1");
-    drop_graphs(b);
     b->Re = Re;
     b->dt = dt;
     b->rtol = rtol;
@@ -1508,12 +1848,14 @@ vip_status vip_3d_set_state(vip_3d* b, const double* u, const double* v, const d
         }
         V3_CUDA(alloc(b->state_bufs, &b->p, N));
         V3_CUDA(alloc(b->state_bufs, &b->phi, N + 1));
-        for (int k = 0; k < 8; ++k) V3_CUDA(alloc(b->state_bufs, &b->kv[k], N + 1));
-        V3_CUDA(alloc(b->state_bufs, &b->dpart, 2 * std::max<int64_t>(DOT_B, (N + 1 + 255) / 256)));
-        V3_CUDA(alloc(b->state_bufs, &b->dres, 2));
-        KS* ksp = nullptr;
-        V3_CUDA(alloc(b->state_bufs, &ksp, 1));
-        b->ks = ksp;
+        for (int c = 0; c < 3; ++c) {
+            V3_CUDA(alloc(b->state_bufs, &b->rhs[c], N + 1));
+            V3_CUDA(alloc(b->state_bufs, &b->gather[0][c], N + 1));
+            V3_CUDA(alloc(b->state_bufs, &b->gather[1][c], N + 1));
+        }
+        V3_CUDA(alloc(b->state_bufs, &b->dpart, (size_t)2 * 9 * b->sms));
+        V3_CUDA(alloc(b->state_bufs, &b->dout, 4));
+        V3_CUDA(alloc(b->state_bufs, &b->dbar, 2));
     }
     const double* src[4] = {u, v, w, p};
     double* dst[4] = {b->vel[0], b->vel[1], b->vel[2], b->p};
@@ -1537,8 +1879,7 @@ vip_status vip_3d_step(vip_3d* b, int32_t nsteps) {
     if (b->k0 < 0) return fail(b, VIP_ERR_ARG, "the 3D step needs an interior node");
     if (nsteps < 0) return fail(b, VIP_ERR_ARG, "nsteps must be >= 0");
     DeviceScope ds(b->device);
-    const int need[5] = {VIP3_OP_LAPLACE, VIP3_OP_GX, VIP3_OP_GY, VIP3_OP_GZ, VIP3_OP_NEUMANN};
-    for (int op : need) V3_TRY(assemble(b, op));
+    V3_TRY(slice_tables(b));
     for (int k = 0; k < nsteps; ++k) V3_TRY(step_once(b));
     return VIP_OK;
 }
