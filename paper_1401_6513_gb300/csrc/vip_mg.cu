@@ -210,9 +210,276 @@ vip_status mg_set_params(vip_ctx* c, Multigrid& M, float omega, float corr) {
     return VIP_OK;
 }
 
-// Dense inverse of one geometry's coarsest operator, A (m x m, row-major), by
-// Gauss-Jordan elimination with partial pivoting in FP64 on the host (setup only;
-// the row updates of each pivot step run on the host's cores with OpenMP).
+// ---- dense inverses of the coarsest operators -------------------------------------------
+//
+// Small ones (HOST_INVERSE cells, every closed geometry) are inverted on the host, larger ones
+// on the device.  There the operator is a band matrix: a cell couples to cells at most two
+// away, so with the cells numbered along the shorter side of the lattice the half bandwidth b
+// is about twice that side (68 of 2,145 unknowns on a 65 x 33 lattice).  Band LU with partial
+// pivoting costs m b^2 operations and m columns of substitution 3 m^2 b, against 2 m^3 for
+// Gauss-Jordan, which neither the host (290 ms at 2,145 cells) nor the FP64 unit (17 ms at
+// its peak) can hide.  All in FP64, with the pivoting that the host's elimination has.
+constexpr int HOST_INVERSE = 64;   // 64 cells: 0.13 ms on the host, 0.20 ms on the device
+
+struct BandMat {
+    int64_t ab, x, inv, c0;   // offsets of the band, the columns of the inverse, the result; first cell
+    int64_t row;              // offset of the geometry's per-row arrays
+    int m, b, ld;             // unknowns, half bandwidth, column stride of the band (3 b + 1)
+};
+
+// Cell r's row of A becomes column pos[r] of the band matrix B = A^T (so that the columns of
+// B's inverse are the rows of A's), B(i, j) at ab[j * ld + 2 b + i - j].  One thread per cell:
+// couplings that coincide (a short periodic side) add up in the order of the stencil.
+__global__ void k_band_fill(const BandMat* __restrict__ mats, int64_t ncell, const double* __restrict__ coef,
+                            const int32_t* __restrict__ nbr, const int32_t* __restrict__ pos,
+                            double* __restrict__ ab) {
+    const BandMat B = mats[blockIdx.y];
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= B.m) return;
+    const int j = pos[B.row + r];
+    double* col = ab + B.ab + (int64_t)j * B.ld + 2 * B.b - j;
+    for (int o = 0; o < 25; ++o) {
+        const int32_t q = nbr[(int64_t)o * ncell + B.c0 + r];
+        if (q >= 0) col[pos[B.row + (q - B.c0)]] += coef[(int64_t)o * ncell + B.c0 + r];
+    }
+    bool empty = true;
+    for (int o = 0; o < 25; ++o) {
+        const int32_t q = nbr[(int64_t)o * ncell + B.c0 + r];
+        if (q >= 0 && col[pos[B.row + (q - B.c0)]] != 0.0) empty = false;
+    }
+    if (empty) col[j] = 1.0;
+}
+
+// Band LU with partial pivoting, one block per geometry.  At step k every warp exchanges rows
+// k and p of its columns and subtracts the multiples of row k from the b rows below; warp 0
+// takes column k + 1 alone, then looks for its pivot and scales it, so that a step needs one
+// barrier and the search and the division run beside the update.  ju is the last column that
+// the pivot rows so far reach (b beyond the diagonal while no rows are exchanged); top[j] the
+// first row of U's column j.  Bound by the FP64 unit of one SM (b^2 multiply-adds a step,
+// 1.2 us at b = 68) and the step's latency: 5.1 ms for 2,145 unknowns.
+__global__ void __launch_bounds__(512) k_band_factor(const BandMat* __restrict__ mats, double* ab, int32_t* piv,
+                                                     int32_t* top, double* udi) {
+    const BandMat B = mats[blockIdx.x];
+    const int m = B.m, b = B.b, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int ld = B.ld;
+    double* M = ab + B.ab + 2 * b;                     // B(i, j) = M[j * (ld - 1) + i]
+    const int64_t cs = ld - 1;
+    __shared__ int s_p[2], s_ju[2];
+    int ju = -1;
+    for (int k = -1; k < m - 1; ++k) {
+        const int p = k >= 0 ? s_p[k & 1] : 0;
+        if (k >= 0) ju = s_ju[k & 1];
+        const int nb = min(b, m - 1 - k);              // rows k + 1 .. k + nb
+        const double* l = M + k * cs + k + 1;
+        if (warp == 0) {
+            const int j = k + 1;
+            double* cj = M + j * cs;
+            if (j <= ju) {
+                const double c = cj[p], a = cj[k];
+                __syncwarp();
+                if (lane == 0 && p != k) { cj[k] = c; cj[p] = a; }
+                __syncwarp();
+                if (c != 0.0)
+                    for (int i = lane; i < nb; i += 32) cj[k + 1 + i] -= l[i] * c;
+                __syncwarp();
+            }
+            // pivot of column j: the first of the largest entries on and below the diagonal
+            const int nj = min(b, m - 1 - j);
+            long long best = -1;
+            int bi = j;
+            for (int i = lane; i <= nj; i += 32) {
+                const long long v = __double_as_longlong(fabs(cj[j + i]));
+                if (v > best) { best = v; bi = j + i; }
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                const long long v = __shfl_xor_sync(0xffffffffu, best, o);
+                const int vi = __shfl_xor_sync(0xffffffffu, bi, o);
+                if (v > best || (v == best && vi < bi)) { best = v; bi = vi; }
+            }
+            const double d = cj[bi], old = cj[j];
+            const double di = fabs(d) > 1e-300 ? 1.0 / d : 0.0;
+            __syncwarp();
+            if (lane == 0 && bi != j) { cj[j] = d; cj[bi] = old; }
+            __syncwarp();
+            for (int i = 1 + lane; i <= nj; i += 32) cj[j + i] *= di;
+            const int ju2 = max(ju, min(bi + b, m - 1));
+            for (int q = ju + 1 + lane; q <= ju2; q += 32) top[B.row + q] = j;
+            if (lane == 0) {
+                piv[B.row + j] = bi;
+                udi[B.row + j] = di;
+                s_p[j & 1] = bi;
+                s_ju[j & 1] = ju2;
+            }
+        } else if (k >= 0 && k + 2 <= ju) {
+            // columns k + 2 .. ju, split over warps 1 .. 15; a warp's columns as one list of elements
+            const int nc = ju - k - 1, per = (nc + 14) / 15;
+            const int j0 = k + 2 + (warp - 1) * per, jn = min(per, ju + 1 - j0);
+            for (int q0 = 0; q0 < jn; q0 += 32) {      // 32 columns at a time (one, unless b > 160)
+                const int qn = min(32, jn - q0);
+                double c = 0.0;
+                if (lane < qn) {
+                    double* cj = M + (j0 + q0 + lane) * cs;
+                    c = cj[p];
+                    if (p != k) {
+                        const double a = cj[k];
+                        cj[k] = c;
+                        cj[p] = a;
+                    }
+                }
+                __syncwarp();
+                int q = 0, i = lane;
+                const int n = qn * nb;
+                for (int e0 = 0; e0 < n; e0 += 32) {
+                    while (i >= nb && q < qn) { i -= nb; ++q; }
+                    const double cq = __shfl_sync(0xffffffffu, c, q & 31);
+                    if (q < qn) M[(j0 + q0 + q) * cs + k + 1 + i] -= l[i] * cq;
+                    i += 32;
+                }
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// Columns of B's inverse by substitution, one warp per column j of the unit matrix: forward
+// from the first step that can reach j, back through U's columns.  3 m^2 b multiply-adds,
+// bound by the FP64 unit and the latency of a step: 3.3 ms for 2,145 unknowns.  The columns of a block are far
+// apart: those at the front take twice the steps of those at the end.
+__global__ void __launch_bounds__(512) k_band_solve(const BandMat* __restrict__ mats, const double* __restrict__ ab,
+                                                    const int32_t* __restrict__ piv, const int32_t* __restrict__ top,
+                                                    const double* __restrict__ udi, double* x) {
+    const BandMat B = mats[blockIdx.y];
+    const int m = B.m, b = B.b, lane = threadIdx.x & 31;
+    const int j = blockIdx.x + (threadIdx.x >> 5) * gridDim.x;
+    if (j >= m) return;
+    const double* M = ab + B.ab + 2 * b;
+    const int64_t cs = B.ld - 1;
+    double* X = x + B.x + (int64_t)j * m;
+    for (int i = lane; i < m; i += 32) X[i] = i == j ? 1.0 : 0.0;
+    __syncwarp();
+    for (int k = max(0, j - b); k < m; ++k) {
+        const int p = piv[B.row + k];
+        const double c = X[p], a = X[k];
+        __syncwarp();
+        if (lane == 0 && p != k) { X[k] = c; X[p] = a; }
+        __syncwarp();
+        const int nb = min(b, m - 1 - k);
+        const double* l = M + k * cs + k + 1;
+        for (int i = lane; i < nb; i += 32) X[k + 1 + i] -= l[i] * c;
+        __syncwarp();
+    }
+    for (int k = m - 1; k >= 0; --k) {
+        const int t = top[B.row + k];
+        const double c = X[k] * udi[B.row + k];
+        const double* u = M + k * cs;
+        __syncwarp();
+        if (lane == 0) X[k] = c;
+        for (int i = t + lane; i < k; i += 32) X[i] -= u[i] * c;
+        __syncwarp();
+    }
+}
+
+// inv (row-major, cells in lattice order) and its FP32 rounding from the columns of B's inverse.
+__global__ void k_band_store(const BandMat* __restrict__ mats, const int32_t* __restrict__ pos,
+                             const double* __restrict__ x, double* __restrict__ inv, float* __restrict__ inv32) {
+    const BandMat B = mats[blockIdx.y];
+    const int64_t total = (int64_t)B.m * B.m;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int r = (int)(e / B.m), c = (int)(e - (int64_t)r * B.m);
+        const double v = x[B.x + (int64_t)pos[B.row + r] * B.m + pos[B.row + c]];
+        inv[B.inv + e] = v;
+        inv32[B.inv + e] = (float)v;
+    }
+}
+
+// Numbering of an nx x ny lattice with the least bandwidth for the couplings nbr: along x or
+// along y first, the other direction straight or (where it is periodic) folded, so that its
+// two ends meet.  Returns the half bandwidth.
+static int band_order(int nx, int ny, int64_t c0, int64_t ncell, const int32_t* nbr, int32_t* pos) {
+    const int m = nx * ny;
+    std::vector<int32_t> cand(m);
+    int best = -1;
+    for (int k = 0; k < 4; ++k) {
+        const int ns = k & 1 ? nx : ny, nf = k & 1 ? ny : nx;
+        for (int r = 0; r < m; ++r) {
+            const int xx = r % nx, yy = r / nx, f = k & 1 ? yy : xx;
+            int q = k & 1 ? xx : yy;
+            if (k & 2) q = q < (ns + 1) / 2 ? 2 * q : 2 * (ns - 1 - q) + 1;
+            cand[r] = q * nf + f;
+        }
+        int b = 0;
+        for (int o = 0; o < 25; ++o)
+            for (int r = 0; r < m; ++r) {
+                const int32_t q = nbr[(int64_t)o * ncell + c0 + r];
+                if (q >= 0) b = std::max(b, std::abs(cand[r] - cand[q - c0]));
+            }
+        if (best < 0 || b < best) {
+            best = b;
+            std::copy(cand.begin(), cand.end(), pos);
+        }
+    }
+    return best;
+}
+
+// Inverses of the geometries listed in mats (m, c0 and inv set), into M.cinv and M.cinv32; as
+// many at a time as keep the temporary columns and bands within 1 GiB (one at least).
+static vip_status band_inverses(vip_ctx* c, Multigrid& M, const MgLevel& lc, std::vector<BandMat> mats,
+                                const std::vector<int2>& dims, const int32_t* hnbr) {
+    cudaStream_t st = c->stream;
+    int64_t rows = 0;
+    for (BandMat& B : mats) { B.row = rows; rows += B.m; }
+    std::vector<int32_t> pos(rows);
+    for (size_t i = 0; i < mats.size(); ++i) {
+        BandMat& B = mats[i];
+        B.b = band_order(dims[i].x, dims[i].y, B.c0, lc.n, hnbr, pos.data() + B.row);
+        B.ld = 3 * B.b + 1;
+    }
+    constexpr int64_t LIMIT = (int64_t)1 << 27;   // doubles
+    struct Tmp {
+        void* p = nullptr;
+        ~Tmp() { cudaFree(p); }
+    };
+    for (size_t g0 = 0, g1; g0 < mats.size(); g0 = g1) {
+        int64_t nab = 0, nx = 0, r0 = mats[g0].row, nr = 0;
+        int mmax = 0;
+        for (g1 = g0; g1 < mats.size() && g1 - g0 < 65535; ++g1) {
+            BandMat& B = mats[g1];
+            const int64_t a = (int64_t)B.m * B.ld, q = (int64_t)B.m * B.m;
+            if (g1 > g0 && nab + nx + a + q > LIMIT) break;
+            B.ab = nab; B.x = nx; B.row -= r0;
+            nab += a; nx += q; nr += B.m;
+            mmax = std::max(mmax, B.m);
+        }
+        const int n = (int)(g1 - g0);
+        // one allocation: matrices, bands, columns, reciprocal pivots, three integer arrays
+        const int64_t db = ((int64_t)n * sizeof(BandMat) + 255) / 256 * 256;
+        Tmp t;
+        VIP_CUDA(cudaMalloc(&t.p, db + (nab + nx + nr) * 8 + 3 * nr * 4));
+        BandMat* dm = (BandMat*)t.p;
+        double* ab = (double*)((char*)t.p + db);
+        double *x = ab + nab, *udi = x + nx;
+        int32_t *dpos = (int32_t*)(udi + nr), *piv = dpos + nr, *top = piv + nr;
+        VIP_CUDA(cudaMemcpyAsync(dm, mats.data() + g0, n * sizeof(BandMat), cudaMemcpyHostToDevice, st));
+        VIP_CUDA(cudaMemcpyAsync(dpos, pos.data() + r0, nr * 4, cudaMemcpyHostToDevice, st));
+        VIP_CUDA(cudaMemsetAsync(ab, 0, nab * 8, st));
+        k_band_fill<<<dim3((mmax + 127) / 128, n), 128, 0, st>>>(dm, lc.n, lc.coef, lc.nbr, dpos, ab);
+        VIP_CUDA(cudaGetLastError());
+        k_band_factor<<<n, 512, 0, st>>>(dm, ab, piv, top, udi);
+        VIP_CUDA(cudaGetLastError());
+        k_band_solve<<<dim3((mmax + 15) / 16, n), 512, 0, st>>>(dm, ab, piv, top, udi, x);
+        VIP_CUDA(cudaGetLastError());
+        k_band_store<<<dim3((unsigned)std::min<int64_t>(((int64_t)mmax * mmax + 255) / 256, 1024), n), 256, 0, st>>>(
+            dm, dpos, x, M.cinv, M.cinv32);
+        VIP_CUDA(cudaGetLastError());
+        VIP_CUDA(cudaStreamSynchronize(st));
+    }
+    return VIP_OK;
+}
+
+// Dense inverse of one small operator, A (m x m, row-major), by
+// Gauss-Jordan elimination with partial pivoting in FP64 on the host (setup only).
 // Cells without a row (empty cells) are decoupled: their unknown stays 0.  The
 // result is stored row-major, inv[i * m + j] = (A^{-1})_{ij}.
 static void coarse_inverse(std::vector<double>& A, int m, double* inv) {
@@ -238,7 +505,6 @@ static void coarse_inverse(std::vector<double>& A, int m, double* inv) {
         double* rk = &T[(size_t)k * w];
         for (int j = 0; j < w; ++j) rk[j] *= di;
         double* t0 = T.data();
-#pragma omp parallel for schedule(static) if (m >= 256)
         for (int i = 0; i < m; ++i) {
             if (i == k) continue;
             double* ri = t0 + (size_t)i * w;
@@ -475,26 +741,39 @@ vip_status mg_build(vip_ctx* c, Multigrid& M) {
         VIP_CUDA(cudaMemcpyAsync(hcoef.data(), lc.coef, hcoef.size() * 8, cudaMemcpyDeviceToHost, st));
         VIP_CUDA(cudaMemcpyAsync(hnbr.data(), lc.nbr, hnbr.size() * 4, cudaMemcpyDeviceToHost, st));
         VIP_CUDA(cudaStreamSynchronize(st));
-        std::vector<double> hinv((size_t)tot);
+        M.cinv_entries = tot;
+        VIP_CUDA(dalloc(c, &M.cinv, tot));
+        VIP_CUDA(dalloc(c, &M.cinv_off, G));
+        VIP_CUDA(dalloc(c, &M.cinv32, tot));
+        VIP_CUDA(cudaMemcpyAsync(M.cinv_off, ioff.data(), G * 8, cudaMemcpyHostToDevice, st));
+        std::vector<BandMat> mats;
+        std::vector<int2> dims;
         for (int g = 0; g < G; ++g) {
             const int m = hg[g].nx[L] * hg[g].ny[L];
             const int64_t c0 = offs[L][g];  // cells numbered densely on the coarsest level
-            std::vector<double> Ad((size_t)m * m, 0.0);
+            if (m > HOST_INVERSE) {
+                mats.push_back({0, 0, ioff[g], c0, 0, m, 0, 0});
+                dims.push_back(make_int2(hg[g].nx[L], hg[g].ny[L]));
+                continue;
+            }
+            std::vector<double> Ad((size_t)m * m, 0.0), inv((size_t)m * m);
+            std::vector<float> inv32((size_t)m * m);
             for (int r = 0; r < m; ++r)
                 for (int o = 0; o < 25; ++o) {
                     const int32_t j = hnbr[(size_t)o * lc.n + c0 + r];
                     if (j >= 0) Ad[(size_t)r * m + (j - c0)] += hcoef[(size_t)o * lc.n + c0 + r];
                 }
-            coarse_inverse(Ad, m, hinv.data() + ioff[g]);
+            coarse_inverse(Ad, m, inv.data());
+            for (size_t i = 0; i < inv.size(); ++i) inv32[i] = (float)inv[i];
+            VIP_CUDA(cudaMemcpyAsync(M.cinv + ioff[g], inv.data(), inv.size() * 8, cudaMemcpyHostToDevice, st));
+            VIP_CUDA(cudaMemcpyAsync(M.cinv32 + ioff[g], inv32.data(), inv32.size() * 4, cudaMemcpyHostToDevice,
+                                     st));
+            VIP_CUDA(cudaStreamSynchronize(st));
         }
-        M.cinv_entries = tot;
-        VIP_CUDA(dalloc(c, &M.cinv, tot));
-        VIP_CUDA(dalloc(c, &M.cinv_off, G));
-        VIP_CUDA(cudaMemcpyAsync(M.cinv, hinv.data(), tot * 8, cudaMemcpyHostToDevice, st));
-        VIP_CUDA(cudaMemcpyAsync(M.cinv_off, ioff.data(), G * 8, cudaMemcpyHostToDevice, st));
-        VIP_CUDA(dalloc(c, &M.cinv32, tot));
-        k_mg_f32<<<(unsigned)((tot + TB - 1) / TB), TB, 0, st>>>(tot, M.cinv, M.cinv32);
-        VIP_CUDA(cudaGetLastError());
+        if (!mats.empty()) {
+            const vip_status s = band_inverses(c, M, lc, mats, dims, hnbr.data());
+            if (s != VIP_OK) return s;
+        }
         VIP_CUDA(cudaStreamSynchronize(st));
         M.ngeom = G;
     }

@@ -17,8 +17,9 @@
 // iteration is five phases between grid barriers (0.9 us each, every wait bounded: 2 s, then
 // VIP_ERR_TIMEOUT), three of them with a reduction (about 2 us, a chain of dependent FP64
 // additions), and is bound by those and by the FP64 unit.  131,072 rows of 5 entries: 57 ->
-// 23 us per iteration (25 with 256 or 1,024 threads a block; before: four blocks per SM meeting at a barrier that slept, CSR rows
-// read by one thread each from memory, six phases).
+// 23 us per iteration (25 with 256 or 1,024 threads a block; before:
+// four blocks per SM meeting at a barrier that slept, CSR rows read by one thread each from
+// memory, six phases).
 #include <cuda_runtime.h>
 
 #include <algorithm>
