@@ -87,6 +87,58 @@ vip_status gather_out(vip_ctx* c, const double* src_padded, double* dst) {
     return VIP_OK;
 }
 
+// 4 R doubles for one call's vectors in padded row order.  Up to STAGE_KEEP bytes the buffer
+// belongs to the context and stays for its next call (cudaMalloc and cudaFree cost 0.1 to 0.5 ms
+// a call, more than applying an operator to 500,000 rows); a larger one is freed with the call.
+// The context's buffer is locked while a call uses it; each such call ends with a wait for the
+// stream, so none is given on while kernels still read it.
+constexpr size_t STAGE_KEEP = (size_t)128 << 20;
+struct StageBuf {
+    double* p = nullptr;
+    bool own = false;
+    std::unique_lock<std::mutex> lock;
+    cudaStream_t st = nullptr;
+    cudaError_t get(vip_ctx* c) {
+        const size_t bytes = (size_t)4 * c->R * sizeof(double);
+        st = c->stream;
+        if (bytes > STAGE_KEEP) {
+            own = true;
+            return cudaMalloc(&p, bytes);
+        }
+        lock = std::unique_lock<std::mutex>(c->stage_mutex);
+        if (!c->stage) {
+            const cudaError_t e = cudaMalloc(&c->stage, bytes);
+            if (e != cudaSuccess) {
+                c->stage = nullptr;
+                return e;
+            }
+        }
+        p = c->stage;
+        return cudaSuccess;
+    }
+    ~StageBuf() {
+        if (p) cudaStreamSynchronize(st);  // early returns
+        if (own) cudaFree(p);
+    }
+};
+
+// Can a kernel on the context's device read x and write y, n entries each, in place of the
+// caller's arrays?  Both lie in this device's memory from the first to the last entry, are
+// aligned as doubles, and do not overlap.  Host arrays and other devices' go through a StageBuf.
+bool direct_vectors(const vip_ctx* c, const double* x, const double* y, int64_t n) {
+    if (n <= 0 || (reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) % sizeof(double)) return false;
+    if (x < y + n && y < x + n) return false;
+    for (const double* p : {x, x + n - 1, y, y + n - 1}) {
+        cudaPointerAttributes a;
+        if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (a.type != cudaMemoryTypeDevice || a.device != c->device) return false;
+    }
+    return true;
+}
+
 vip_status do_step(vip_ctx* c, cudaStream_t s) {
     VIP_CUDA(cudaEventRecord(c->ev[0], s));
     launch_conv_rhs(c, s);
@@ -148,6 +200,7 @@ void vip_destroy(vip_ctx* c) {
     if (c->graph) cudaGraphExecDestroy(c->graph);
     cudaStreamSynchronize(c->stream);
     for (void* p : c->allocs) cudaFree(p);
+    cudaFree(c->stage);
     cnn_free(c);
     for (int i = 0; i <= VIP_PHASE_COUNT; ++i)
         if (c->ev[i]) cudaEventDestroy(c->ev[i]);
@@ -414,6 +467,7 @@ vip_status vip_build(vip_ctx* c) {
     std::vector<int32_t> prg(R, 0), first(G);
     std::vector<int8_t> prt(R, ROW_PAD);
     std::vector<GeomDev> gd(G);
+    int64_t mu = 0;
     for (int gi = 0; gi < G; ++gi) {
         const Geom& g = c->geoms[gi];
         for (int64_t i = 0; i < g.n; ++i) {
@@ -431,7 +485,7 @@ vip_status vip_build(vip_ctx* c) {
             if (pin < 0) return fail(c, VIP_ERR_ARG, "a closed geometry needs an interior node");
         }
         gd[gi] = GeomDev{g.row0, g.nrows, g.n, g.Lx, g.Ly, g.Re, g.dt, g.dt / (2.0 * g.Re),
-                         g.bordered ? 1 : 0, pin, g.probes};
+                         g.bordered ? 1 : 0, pin, g.probes, g.off, g.bordered ? c->N + mu++ : -1};
         if (g.probes == VIP_PROBES_INSIDE && !(c->support > 2.0))
             return fail(c, VIP_ERR_ARG, "VIP_PROBES_INSIDE needs a support ratio above 2");
     }
@@ -904,14 +958,22 @@ vip_status vip_apply(vip_ctx* c, int which, const double* x, double* y) {
         case VIP_OP_POISSON: S = c->T.pois; break;
         default: return fail(c, VIP_ERR_ARG, "unknown table");
     }
-    double *xp = nullptr, *yp = nullptr;
-    VIP_CUDA(cudaMalloc(&xp, 2 * R * 8));
-    VIP_CUDA(cudaMalloc(&yp, 2 * R * 8));
-    cudaStream_t st = c->stream;
-    VIP_CUDA(cudaMemsetAsync(xp, 0, 2 * R * 8, st));
+    const bool pois = which == VIP_OP_POISSON;
     if (which == VIP_OP_HELM_V) off = R;
+    cudaStream_t st = c->stream;
+    const int64_t nvec = c->N + (pois ? c->nbordered : 0);
+    if (direct_vectors(c, x, y, nvec)) {
+        launch_apply(c, S, off, pois, x, y, st);
+        VIP_CUDA(cudaGetLastError());
+        VIP_CUDA(cudaStreamSynchronize(st));
+        return VIP_OK;
+    }
+    StageBuf buf;
+    VIP_CUDA(buf.get(c));
+    double *xp = buf.p, *yp = buf.p + 2 * R;
+    VIP_CUDA(cudaMemsetAsync(xp, 0, 2 * R * 8, st));
     vip_status s = scatter(c, x, xp + off);
-    if (s == VIP_OK && which == VIP_OP_POISSON) {  // mu entries
+    if (s == VIP_OK && pois) {  // mu entries
         int64_t k = 0;
         for (const Geom& g : c->geoms)
             if (g.bordered) {
@@ -922,7 +984,7 @@ vip_status vip_apply(vip_ctx* c, int which, const double* x, double* y) {
     if (s == VIP_OK) {
         launch_spmv(S, xp, yp, st);
         s = gather_out(c, yp + off, y);
-        if (s == VIP_OK && which == VIP_OP_POISSON) {
+        if (s == VIP_OK && pois) {
             int64_t k = 0;
             for (const Geom& g : c->geoms)
                 if (g.bordered) {
@@ -932,8 +994,6 @@ vip_status vip_apply(vip_ctx* c, int which, const double* x, double* y) {
         }
     }
     cudaError_t e = cudaStreamSynchronize(st);
-    cudaFree(xp);
-    cudaFree(yp);
     if (s != VIP_OK) return s;
     if (e != cudaSuccess) return fail(c, VIP_ERR_CUDA, cudaGetErrorString(e));
     return VIP_OK;
@@ -943,8 +1003,9 @@ vip_status vip_convection(vip_ctx* c, const double* u, const double* v, double* 
     if (!c || !u || !v || !Nu || !Nv) return VIP_ERR_ARG;
     if (!c->built) return fail(c, VIP_ERR_ARG, "vip_convection before vip_build");
     const int64_t R = c->R;
-    double* buf = nullptr;
-    VIP_CUDA(cudaMalloc(&buf, 4 * R * 8));
+    StageBuf stage;
+    VIP_CUDA(stage.get(c));
+    double* buf = stage.p;
     cudaStream_t st = c->stream;
     VIP_CUDA(cudaMemsetAsync(buf, 0, 4 * R * 8, st));
     vip_status s = scatter(c, u, buf);
@@ -955,7 +1016,6 @@ vip_status vip_convection(vip_ctx* c, const double* u, const double* v, double* 
         if (s == VIP_OK) s = gather_out(c, buf + 3 * R, Nv);
     }
     cudaError_t e = cudaStreamSynchronize(st);
-    cudaFree(buf);
     if (s != VIP_OK) return s;
     if (e != cudaSuccess) return fail(c, VIP_ERR_CUDA, cudaGetErrorString(e));
     return VIP_OK;
@@ -972,12 +1032,11 @@ vip_status vip_solve(vip_ctx* c, int which, const double* b, double* x, int prec
     if (!(rtol > 0.0)) return fail(c, VIP_ERR_ARG, "bad rtol");
     const int64_t R = c->R;
     bool pois = which == VIP_OP_POISSON;
-    double *bp = nullptr, *xp = nullptr;
-    VIP_CUDA(cudaMalloc(&bp, 2 * R * 8));
-    VIP_CUDA(cudaMalloc(&xp, 2 * R * 8));
+    StageBuf buf;
+    VIP_CUDA(buf.get(c));
+    double *bp = buf.p, *xp = buf.p + 2 * R;
     cudaStream_t st = c->stream;
-    VIP_CUDA(cudaMemsetAsync(bp, 0, 2 * R * 8, st));
-    VIP_CUDA(cudaMemsetAsync(xp, 0, 2 * R * 8, st));
+    VIP_CUDA(cudaMemsetAsync(bp, 0, 4 * R * 8, st));
     VIP_CUDA(cudaMemsetAsync(c->d_status, 0, 4, st));
     int64_t off = which == VIP_OP_HELM_V ? R : 0;
     vip_status s = scatter(c, b, bp + off);
@@ -1011,8 +1070,6 @@ vip_status vip_solve(vip_ctx* c, int which, const double* b, double* x, int prec
     cudaMemcpyAsync(rr.data(), P.out_relres, P.nsys * 8, cudaMemcpyDeviceToHost, st);
     cudaMemcpyAsync(&hs, c->d_status, 4, cudaMemcpyDeviceToHost, st);
     cudaError_t e = cudaStreamSynchronize(st);
-    cudaFree(bp);
-    cudaFree(xp);
     if (s != VIP_OK) return s;
     if (e != cudaSuccess) return fail(c, VIP_ERR_CUDA, cudaGetErrorString(e));
     int32_t mi = 0;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -85,6 +86,8 @@ struct GeomDev {
     int32_t bordered;
     int64_t pin;       // bordered: padded row of the reference node k (first interior node)
     int32_t probes;    // VIP_PROBES_*
+    int64_t off;       // first node in caller order
+    int64_t mu;        // bordered: place of mu in a caller's vector (behind all nodes)
 };
 
 // Work split of a persistent Krylov launch over a batch of systems.
@@ -204,6 +207,9 @@ struct vip_ctx {
     double prof_ms[VIP_PHASE_COUNT] = {0, 0, 0, 0, 0};
     int64_t prof_steps = 0;
     std::vector<void*> allocs;
+    // staging vectors of the calls that take caller-order arrays (StageBuf), kept between calls
+    std::mutex stage_mutex;
+    double* stage = nullptr;
 };
 
 namespace vip {
@@ -237,6 +243,8 @@ void launch_conv_rhs(vip_ctx* c, cudaStream_t s);
 void launch_div(vip_ctx* c, cudaStream_t s);
 void launch_project(vip_ctx* c, cudaStream_t s);
 void launch_spmv(const Sell& A, const double* x, double* y, cudaStream_t s);
+void launch_apply(vip_ctx* c, const Sell& A, int64_t row_off, bool with_mu, const double* x, double* y,
+                  cudaStream_t s);
 void launch_convection(vip_ctx* c, const double* u, const double* v, double* Nu, double* Nv,
                        cudaStream_t s);
 // Device scratch that outlives no call: freed on every return path (cudaFree waits

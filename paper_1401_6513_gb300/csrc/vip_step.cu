@@ -163,6 +163,61 @@ __global__ void k_spmv(Sell A, const double* __restrict__ x, double* __restrict_
     y[r] = gather(A, r, x);
 }
 
+// y = A x between vectors in caller order: node row r of geometry g is node r - row0 + off, so
+// a row's columns map by one shift, and mu (its border row) lies behind all nodes.  row_off:
+// first row of the system in a table that holds several.  The sum is k_spmv's (same entries,
+// same order).  Bound by the table's bytes and the FP64 unit alike (525,313 rows of 18 entries:
+// 17 us each), so the next four entries' columns and values are under way while four are
+// gathered and added: the h = 1/32 channel's five operators take 43 us a call with its launch
+// and wait (74 without running ahead; eight entries ahead 46, 12 blocks of fewer registers 58;
+// 270 through padded copies in buffers allocated for the call).
+constexpr int APPLY_THREADS = 128, APPLY_U = 4, APPLY_BLOCKS = 8;
+__global__ void __launch_bounds__(APPLY_THREADS, APPLY_BLOCKS)
+    k_apply(Sell A, int64_t R, int64_t row_off, int with_mu, const int8_t* __restrict__ row_type,
+            const int32_t* __restrict__ row_geom, const GeomDev* __restrict__ gdev, const double* __restrict__ x,
+            double* __restrict__ y) {
+    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= R) return;
+    const int rt = row_type[r];
+    const GeomDev& G = gdev[row_geom[r]];
+    const int64_t q = row_off + r, s = q >> 5;
+    const int64_t base = A.sptr[s] + (q & 31);
+    const int w = A.width[s];
+    if (rt != ROW_NODE && !(rt == ROW_BORDER && with_mu)) return;
+    const double* xs = x + (G.off - G.row0 - row_off);   // entry of table column c: xs[c]
+    const int64_t mu = G.mu;
+    const int border = G.bordered && with_mu ? (int)(row_off + G.row0 + G.n) : -1;
+    const int32_t* pc = A.col + base;
+    const double* pv = A.v64 + base;
+    constexpr int U = APPLY_U;
+    int col[U];
+    double a[U];
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (k0 + k < w) {
+                col[k] = __ldg(pc + (k0 + k) * SLICE);
+                a[k] = __ldg(pv + (k0 + k) * SLICE);
+            }
+    };
+    double sum = 0.0;
+    load(0);
+    for (int k0 = 0; k0 < w; k0 += U) {
+        double f[U], b[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (k0 + k < w) {
+                f[k] = __ldg(col[k] == border ? x + mu : xs + col[k]);
+                b[k] = a[k];
+            }
+        load(k0 + U);
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (k0 + k < w) sum += b[k] * f[k];
+    }
+    y[rt == ROW_BORDER ? mu : r + G.off - G.row0] = sum;
+}
+
 __global__ void k_convection(StepArgs a, const double* __restrict__ u, const double* __restrict__ v,
                              double* __restrict__ Nu, double* __restrict__ Nv) {
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -198,6 +253,11 @@ void launch_div(vip_ctx* c, cudaStream_t s) {
 void launch_project(vip_ctx* c, cudaStream_t s) {
     k_project<<<nblk(c->R, 256), 256, 0, s>>>(step_args(c), c->hsol, c->phi, c->u, c->v, c->p,
                                               c->d_step, c->uv_prev);
+}
+void launch_apply(vip_ctx* c, const Sell& A, int64_t row_off, bool with_mu, const double* x, double* y,
+                  cudaStream_t s) {
+    k_apply<<<nblk(c->R, APPLY_THREADS), APPLY_THREADS, 0, s>>>(A, c->R, row_off, with_mu ? 1 : 0, c->row_type, c->row_geom, c->gdev,
+                                            x, y);
 }
 void launch_spmv(const Sell& A, const double* x, double* y, cudaStream_t s) {
     k_spmv<<<nblk(A.nrows, 256), 256, 0, s>>>(A, x, y);
