@@ -228,9 +228,11 @@ __global__ void k_ws_fit(int64_t n, const float* __restrict__ t, const float* __
 // extrapolation a (phi^n - phi^{n-1}) leaves), else t.
 __global__ void k_loss(int64_t n, const float* __restrict__ y, const float* __restrict__ t,
                        const float* __restrict__ dp, double a, const float* __restrict__ m, double inv_cnt,
-                       __nv_bfloat16* __restrict__ gy, double* __restrict__ part) {
+                       const double* __restrict__ inv_dev, __nv_bfloat16* __restrict__ gy,
+                       double* __restrict__ part) {
     __shared__ double s[256];
     double acc = 0.0;
+    if (inv_dev) inv_cnt = *inv_dev;
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x) {
         const double tc = dp ? (double)t[c] - a * (double)dp[c] : (double)t[c];
         double d = (double)m[c] * ((double)y[c] - tc);
@@ -305,15 +307,38 @@ __global__ void k_rloss1(int64_t n, const CnnImage* __restrict__ img, int nimg, 
 __global__ void k_rloss2(int64_t n, const CnnImage* __restrict__ img, int nimg, const float* __restrict__ y,
                          const float* __restrict__ t, const float* __restrict__ dp, double a,
                          const float* __restrict__ m, double lam, const float* __restrict__ q,
-                         double inv_cnt, __nv_bfloat16* __restrict__ gy) {
+                         double inv_cnt, const double* __restrict__ inv_dev, __nv_bfloat16* __restrict__ gy) {
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n) return;
+    if (inv_dev) inv_cnt = *inv_dev;
     const CnnImage I = img[cnn_image_of(img, nimg, c)];
     const double lq = cnn_nbr_sum(I, c, [&](int64_t j) { return (double)q[j]; }) - 4.0 * (double)q[c];
     const double g = 2.0 * (double)m[c] * (lq + lam * cnn_err(c, y, t, dp, a, m)) * inv_cnt;
     __nv_bfloat16* o = gy + c * CNN_COUT;
     o[0] = __float2bfloat16((float)g);
     for (int k = 1; k < CNN_COUT; ++k) o[k] = __float2bfloat16(0.0f);
+}
+
+// vip_ws_eval: the FP32 input rounded to BF16, four entries a thread (n: a multiple of 16)
+__global__ void k_ws_input(int64_t n4, const float4* __restrict__ x, uint2* __restrict__ out) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n4) return;
+    const float4 v = __ldcs(x + i);
+    __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+    out[i] = make_uint2(*reinterpret_cast<uint32_t*>(&lo), *reinterpret_cast<uint32_t*>(&hi));
+}
+
+// cells with a nonzero mask, and the reciprocal of their number (at least 1) that the loss
+// kernels take from the device
+__global__ void k_ws_count(int64_t n, const float* __restrict__ m, unsigned long long* __restrict__ cnt) {
+    int k = 0;
+    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x)
+        k += m[c] != 0.0f;
+    k = __reduce_add_sync(0xffffffffu, k);
+    if ((threadIdx.x & 31) == 0 && k) atomicAdd(cnt, (unsigned long long)k);
+}
+__global__ void k_ws_inv(const unsigned long long* __restrict__ cnt, double* __restrict__ inv) {
+    *inv = 1.0 / fmax((double)*cnt, 1.0);
 }
 
 // sum block partials in block order into the gradient slots of the layer
@@ -393,6 +418,10 @@ struct Cnn {
     float* s_dprev = nullptr;       // (phi^n - phi^{n-1}) / S of each sample (FP32)
     // test images (vip_cnn_forward / vip_cnn_grads)
     CnnImage* timg = nullptr;
+    // input of vip_ws_eval (BF16, kept and grown like the activations), count of its loss cells
+    __nv_bfloat16* ein = nullptr;
+    int64_t ein_cells = 0;
+    unsigned long long* ecnt = nullptr;   // [2]: the count, the bits of its reciprocal
 };
 
 }  // namespace vip
@@ -513,27 +542,64 @@ vip_status backward(vip_ctx* c, Cnn& N, const CnnImage* img, int nimg, int64_t n
 
 vip_status loss_grad(vip_ctx* c, Cnn& N, const CnnImage* img, int nimg, int64_t n, const float* tgt,
                      const float* dprev, double a, const float* mask, double cnt, double* loss_out,
-                     cudaStream_t s) {
+                     cudaStream_t s, const unsigned long long* cnt_dev = nullptr, const double* inv_dev = nullptr) {
     int nb = N.loss_blocks;
     if (N.loss_kind == 1) {
         k_rloss1<<<nb, 256, 0, s>>>(n, img, nimg, N.out, tgt, dprev, a, mask, N.loss_lam, N.lq, N.loss_part);
         k_rloss2<<<nblk(n, 256), 256, 0, s>>>(n, img, nimg, N.out, tgt, dprev, a, mask, N.loss_lam, N.lq,
-                                              1.0 / std::max(cnt, 1.0), N.gl);
+                                              1.0 / std::max(cnt, 1.0), inv_dev, N.gl);
     } else {
-        k_loss<<<nb, 256, 0, s>>>(n, N.out, tgt, dprev, a, mask, 1.0 / std::max(cnt, 1.0), N.gl,
-                                  N.loss_part);
+        k_loss<<<nb, 256, 0, s>>>(n, N.out, tgt, dprev, a, mask, 1.0 / std::max(cnt, 1.0), inv_dev,
+                                  N.gl, N.loss_part);
     }
     VIP_CUDA(cudaGetLastError());
     if (loss_out) {
         std::vector<double> part(nb);
+        unsigned long long hcnt = 0;
         VIP_CUDA(cudaMemcpyAsync(part.data(), N.loss_part, nb * 8, cudaMemcpyDeviceToHost, s));
+        if (cnt_dev) VIP_CUDA(cudaMemcpyAsync(&hcnt, cnt_dev, 8, cudaMemcpyDeviceToHost, s));
         VIP_CUDA(cudaStreamSynchronize(s));
+        if (cnt_dev) cnt = (double)hcnt;
         double L = 0;
         for (double v : part) L += v;
         *loss_out = L / std::max(cnt, 1.0);
     }
     return VIP_OK;
 }
+
+// A caller's array of n floats on the context's device: the array itself if all of it is this
+// device's memory and 16-byte aligned (the loads of k_ws_input), else a copy for this call.
+struct EvalArray {
+    const float* p = nullptr;
+    float* own = nullptr;
+    cudaStream_t st = nullptr;
+    cudaError_t get(const vip_ctx* c, const float* src, int64_t n, cudaStream_t s) {
+        bool direct = reinterpret_cast<uintptr_t>(src) % 16 == 0;
+        for (const float* q : {src, src + n - 1}) {
+            cudaPointerAttributes a;
+            if (cudaPointerGetAttributes(&a, q) != cudaSuccess) {
+                cudaGetLastError();
+                direct = false;
+            } else {
+                direct = direct && a.type == cudaMemoryTypeDevice && a.device == c->device;
+            }
+        }
+        if (direct) {
+            p = src;
+            return cudaSuccess;
+        }
+        cudaError_t e = cudaMalloc(&own, n * sizeof(float));
+        if (e != cudaSuccess) return e;
+        st = s;
+        p = own;
+        return cudaMemcpyAsync(own, src, n * sizeof(float), cudaMemcpyDefault, s);
+    }
+    ~EvalArray() {
+        if (!own) return;
+        cudaStreamSynchronize(st);
+        cudaFree(own);
+    }
+};
 
 vip_status adam(vip_ctx* c, Cnn& N, double lr, cudaStream_t s) {
     N.adam_t++;
@@ -986,35 +1052,35 @@ vip_status vip_ws_eval(vip_ctx* c, int32_t H, int32_t W, const float* x, float* 
     I.off = 0; I.H = H; I.W = W; I.tile0 = 0;
     VIP_CUDA(cudaMemcpyAsync(N.timg, &I, sizeof(I), cudaMemcpyHostToDevice, s));
     int64_t ntiles = (int64_t)H * ((W + CNN_TILE - 1) / CNN_TILE);
-    // input: FP32 [H][W][16] -> BF16
-    std::vector<float> hx(n * CNN_CIN);
-    VIP_CUDA(cudaMemcpy(hx.data(), x, n * CNN_CIN * 4, cudaMemcpyDefault));
-    std::vector<__nv_bfloat16> hb(n * CNN_CIN);
-    for (int64_t i = 0; i < n * CNN_CIN; ++i) hb[i] = __float2bfloat16(hx[i]);
-    __nv_bfloat16* in = nullptr;
-    VIP_CUDA(cudaMalloc(&in, n * CNN_CIN * 2));
-    VIP_CUDA(cudaMemcpyAsync(in, hb.data(), n * CNN_CIN * 2, cudaMemcpyHostToDevice, s));
+    // input: FP32 [H][W][16] -> BF16, read where it lies if that is this device's memory.  Writers
+    // of the caller's arrays on the default stream have finished, whatever kind of stream s is.
+    VIP_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+    if (N.ein_cells < n) {
+        VIP_CUDA(dalloc(c, &N.ein, n * CNN_CIN));
+        N.ein_cells = n;
+    }
+    if (!N.ecnt) VIP_CUDA(dalloc(c, &N.ecnt, 2));
+    __nv_bfloat16* in = N.ein;
+    EvalArray dx, dt, dm;
+    VIP_CUDA(dx.get(c, x, n * CNN_CIN, s));
+    k_ws_input<<<nblk(n * CNN_CIN / 4, 256), 256, 0, s>>>(n * CNN_CIN / 4, reinterpret_cast<const float4*>(dx.p),
+                                                         reinterpret_cast<uint2*>(in));
+    VIP_CUDA(cudaGetLastError());
     st = forward(c, N, N.timg, 1, ntiles, in, s);
     if (st == VIP_OK && y) VIP_CUDA(cudaMemcpyAsync(y, N.out, n * 4, cudaMemcpyDefault, s));
     if (st == VIP_OK && grads && target && mask) {
-        float *dt = nullptr, *dm = nullptr;
-        VIP_CUDA(cudaMalloc(&dt, n * 4));
-        VIP_CUDA(cudaMalloc(&dm, n * 4));
-        VIP_CUDA(cudaMemcpyAsync(dt, target, n * 4, cudaMemcpyDefault, s));
-        VIP_CUDA(cudaMemcpyAsync(dm, mask, n * 4, cudaMemcpyDefault, s));
-        std::vector<float> hmk(n);
-        VIP_CUDA(cudaMemcpy(hmk.data(), mask, n * 4, cudaMemcpyDefault));
-        double cnt = 0;
-        for (float v : hmk) cnt += v != 0.0f;
-        st = loss_grad(c, N, N.timg, 1, n, dt, nullptr, 0.0, dm, cnt, loss, s);
+        VIP_CUDA(dt.get(c, target, n, s));
+        VIP_CUDA(dm.get(c, mask, n, s));
+        double* inv = reinterpret_cast<double*>(N.ecnt + 1);
+        VIP_CUDA(cudaMemsetAsync(N.ecnt, 0, 8, s));
+        k_ws_count<<<(unsigned)std::min<int64_t>(nblk(n, 256), 1024), 256, 0, s>>>(n, dm.p, N.ecnt);
+        k_ws_inv<<<1, 1, 0, s>>>(N.ecnt, inv);
+        VIP_CUDA(cudaGetLastError());
+        st = loss_grad(c, N, N.timg, 1, n, dt.p, nullptr, 0.0, dm.p, 1.0, loss, s, N.ecnt, inv);
         if (st == VIP_OK) st = backward(c, N, N.timg, 1, ntiles, in, s);
         if (st == VIP_OK) VIP_CUDA(cudaMemcpyAsync(grads, N.grads, N.L.total * 4, cudaMemcpyDefault, s));
-        VIP_CUDA(cudaStreamSynchronize(s));
-        cudaFree(dt);
-        cudaFree(dm);
     }
     cudaError_t e = cudaStreamSynchronize(s);
-    cudaFree(in);
     if (st != VIP_OK) return st;
     if (e != cudaSuccess) return fail(c, VIP_ERR_CUDA, cudaGetErrorString(e));
     int32_t hs = 0;
