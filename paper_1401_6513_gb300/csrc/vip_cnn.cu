@@ -222,6 +222,14 @@ __global__ void k_ws_fit(int64_t n, const float* __restrict__ t, const float* __
     }
 }
 
+// gradient g of cell c's output channel 0, zeros in the MMA's other channels (32 bytes)
+__device__ __forceinline__ void put_gy(__nv_bfloat16* gy, int64_t c, float g) {
+    static_assert(CNN_COUT == 16, "");
+    uint4* o = reinterpret_cast<uint4*>(gy + c * CNN_COUT);
+    o[0] = make_uint4(__bfloat16_as_ushort(__float2bfloat16(g)), 0u, 0u, 0u);
+    o[1] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 // MSE loss and its gradient wrt the output channel 0: gy = 2 (y - t) m / count.
 // Block partials of the loss in fixed order.
 // The target is t - a dp when dp is given (the part of the increment change that the
@@ -237,9 +245,7 @@ __global__ void k_loss(int64_t n, const float* __restrict__ y, const float* __re
         const double tc = dp ? (double)t[c] - a * (double)dp[c] : (double)t[c];
         double d = (double)m[c] * ((double)y[c] - tc);
         acc += d * d;
-        __nv_bfloat16* g = gy + c * CNN_COUT;
-        g[0] = __float2bfloat16((float)(2.0 * d * inv_cnt));
-        for (int k = 1; k < CNN_COUT; ++k) g[k] = __float2bfloat16(0.0f);
+        put_gy(gy, c, (float)(2.0 * d * inv_cnt));
     }
     s[threadIdx.x] = acc;
     __syncthreads();
@@ -272,7 +278,8 @@ __device__ __forceinline__ double cnn_err(int64_t c, const float* __restrict__ y
 template <class F>
 __device__ __forceinline__ double cnn_nbr_sum(const CnnImage& I, int64_t c, F&& f) {
     const int64_t k = c - I.off;
-    const int iy = (int)(k / I.W), ix = (int)(k % I.W);
+    const int iy = k <= 0xffffffffll ? (int)((uint32_t)k / (uint32_t)I.W) : (int)(k / I.W);
+    const int ix = (int)(k - (int64_t)iy * I.W);
     double s = 0.0;
     if (ix > 0) s += f(c - 1);
     if (ix + 1 < I.W) s += f(c + 1);
@@ -314,9 +321,7 @@ __global__ void k_rloss2(int64_t n, const CnnImage* __restrict__ img, int nimg, 
     const CnnImage I = img[cnn_image_of(img, nimg, c)];
     const double lq = cnn_nbr_sum(I, c, [&](int64_t j) { return (double)q[j]; }) - 4.0 * (double)q[c];
     const double g = 2.0 * (double)m[c] * (lq + lam * cnn_err(c, y, t, dp, a, m)) * inv_cnt;
-    __nv_bfloat16* o = gy + c * CNN_COUT;
-    o[0] = __float2bfloat16((float)g);
-    for (int k = 1; k < CNN_COUT; ++k) o[k] = __float2bfloat16(0.0f);
+    put_gy(gy, c, (float)g);
 }
 
 // vip_ws_eval: the FP32 input rounded to BF16, four entries a thread (n: a multiple of 16)
@@ -341,21 +346,28 @@ __global__ void k_ws_inv(const unsigned long long* __restrict__ cnt, double* __r
     *inv = 1.0 / fmax((double)*cnt, 1.0);
 }
 
-// sum block partials in block order into the gradient slots of the layer
-__global__ void k_wgrad_sum(const float* __restrict__ part, int nblocks, int cin, int cout, int creal,
-                            float* __restrict__ gw, float* __restrict__ gb) {
-    const int nent = 9 * cin * cout;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nent + cout; e += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += part[(int64_t)b * (nent + cout) + e];
-        if (e < nent) {
-            int tap = e / (cin * cout);
-            int rem = e - tap * cin * cout;
-            int ci = rem / cout, co = rem % cout;
-            if (co < creal) gw[((int64_t)tap * cin + ci) * creal + co] = (float)s;
-        } else if (e - nent < creal) {
-            gb[e - nent] = (float)s;
-        }
+// Sum the blocks' partials into the gradient slots of the layer, in FP64 and in a fixed order:
+// warp w of a block adds up partials w, w + 8, .. of 32 entries, then the eight sums are added.
+// (One thread per entry took 68 us for 304 partials, a chain of as many dependent additions.)
+__global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ part, int nblocks, int cin, int cout,
+                                                   int creal, float* __restrict__ gw, float* __restrict__ gb) {
+    __shared__ double s_sum[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nent = 9 * cin * cout, e = blockIdx.x * 32 + lane;
+    double s = 0.0;
+    if (e < nent + cout)
+        for (int b = warp; b < nblocks; b += 8) s += part[(int64_t)b * (nent + cout) + e];
+    s_sum[warp][lane] = s;
+    __syncthreads();
+    if (warp != 0 || e >= nent + cout) return;
+    for (int w = 1; w < 8; ++w) s += s_sum[w][lane];
+    if (e < nent) {
+        int tap = e / (cin * cout);
+        int rem = e - tap * cin * cout;
+        int ci = rem / cout, co = rem % cout;
+        if (co < creal) gw[((int64_t)tap * cin + ci) * creal + co] = (float)s;
+    } else if (e - nent < creal) {
+        gb[e - nent] = (float)s;
     }
 }
 
@@ -510,7 +522,7 @@ vip_status backward(vip_ctx* c, Cnn& N, const CnnImage* img, int nimg, int64_t n
             cudaError_t e = cnn_wgrad_tc(wa, nb, s, &why);
             if (e != cudaSuccess) return fail(c, VIP_ERR_CUDA, why);
         }
-        k_wgrad_sum<<<64, 256, 0, s>>>(N.wg_part, nb, cin, cout, N.L.creal[l], N.grads + N.L.w[l],
+        k_wgrad_sum<<<nblk(9 * cin * cout + cout, 32), 256, 0, s>>>(N.wg_part, nb, cin, cout, N.L.creal[l], N.grads + N.L.w[l],
                                        N.grads + N.L.b[l]);
         VIP_CUDA(cudaGetLastError());
         if (l > 0) {  // gradient wrt the pre-activation of layer l-1

@@ -1,24 +1,28 @@
 // 3x3 convolution of the warm-start network as an implicit GEMM on the 5th-generation
 // tensor cores (tcgen05, kind::f16: BF16 x BF16 -> FP32 accumulators in TMEM).
 //
-// A CTA loops over tiles of 128 consecutive pixels of one lattice row (persistent
-// grid).  Per tile it stages the 3 x 130 halo of the input in shared memory,
-// channel-chunk planar: plane[c][row][col] holds channels 8c..8c+7 (16 bytes) of one
-// pixel.  In that layout the 8-pixel x 8-channel core matrices of the MMA operand A
-// are 128 contiguous bytes, so every one of the nine taps is the same operand seen
-// from a shifted start address -- no im2col copy.  The weights sit in shared memory
-// for the whole launch in the same core-matrix layout ([tap][chunk][cout][8 ci]).
-// One thread issues 9 * Cin/16 MMAs (K = 16 each) and commits them to an mbarrier;
-// the four warps then read their 32 TMEM lanes with tcgen05.ld and run the epilogue.
+// A tile is 128 consecutive pixels of one lattice row.  A CTA walks down a strip of 128 columns
+// (a contiguous range of the tiles in strip order), so that of the three input rows of a tile
+// two are already there: rows live in a ring in shared memory, channel-chunk planar --
+// slot[row][c][col] holds channels 8c..8c+7 (16 bytes) of one of 130 pixels.  In that layout the
+// 8-pixel x 8-channel core matrices of the MMA operand A are 128 contiguous bytes, so every one
+// of the nine taps is the same operand seen from a shifted start address -- no im2col copy.  The
+// weights sit in shared memory for the whole launch in the same core-matrix layout
+// ([tap][chunk][cout][8 ci]).  One thread issues 9 * Cin/16 MMAs (K = 16 each) and commits them
+// to an mbarrier; the four warps then read their 32 TMEM lanes with tcgen05.ld and run the
+// epilogue.
 //
-// Pipeline: two halo buffers and two TMEM accumulators.  The halo of a tile is
-// fetched with cp.async (16-byte copies, zero-filled outside the image), so all of a
-// thread's copies are in flight at once, and the tile after next is fetched while
-// the current tile's MMAs run and the previous tile's epilogue drains its
-// accumulator: in iteration k the CTA waits for the MMAs of tile k, issues those of
-// tile k+1 (whose halo landed during iteration k-1), starts the copies of tile k+2
-// into the buffer tile k has released, and then runs tile k's epilogue.  Every
-// mbarrier wait is bounded (2 s, then VIP_ERR_TIMEOUT); TMEM is always freed.
+// Pipeline: a ring of RING rows and two TMEM accumulators.  Rows are fetched with cp.async
+// (16-byte copies, neighbouring threads the chunks of one pixel; zero-filled outside the image)
+// up to three rows ahead.  In iteration k the CTA waits for the MMAs of tile k, issues those of
+// tile k+1, starts the copies of the rows that fit into what tile k has released, and then runs
+// tile k's epilogue.  Every mbarrier wait is bounded (2 s, then VIP_ERR_TIMEOUT); TMEM is always
+// freed.
+//
+// A layer of 32 channels moves 67 MB at 513 x 1025 (10 us) and its MMAs read 4 KB of A each from
+// shared memory (9 us).  It takes 35 to 41 us; 98 when every tile fetched its three rows with copies
+// that touched one chunk of 32 pixels at a time, wrote 16 bytes at a time and read the ReLU mask
+// element by element.
 #include <algorithm>
 #include <cstdio>
 
@@ -27,13 +31,14 @@
 namespace vip {
 
 constexpr int PLANE_COLS = CNN_TILE + 2;               // 130
-constexpr int PLANE_BYTES = 3 * PLANE_COLS * 16;       // 6240
+constexpr int PLANE_BYTES = PLANE_COLS * 16;           // 2080: one row of one chunk
 constexpr int MAX_CHUNKS = CNN_CH / 8;                 // 4
-constexpr int SMEM_IN = MAX_CHUNKS * PLANE_BYTES;      // 24960
+constexpr int SLOT_BYTES = MAX_CHUNKS * PLANE_BYTES;   // 8320: one row
+constexpr int RING = 6;   // rows: a tile's three and, where the next tile starts a new strip, its three
 constexpr int SMEM_W = 9 * MAX_CHUNKS * CNN_CH * 16;   // 18432
-// Two halo buffers, the weights, two mbarriers, the TMEM address word and the
-// failure flag: three CTAs (3 x 64 TMEM columns) per SM.
-constexpr int SMEM_CONV = 2 * SMEM_IN + SMEM_W + 64;
+// The ring, the weights, the bias, two mbarriers and the TMEM address word: three CTAs (3 x 64
+// TMEM columns) per SM.
+constexpr int SMEM_CONV = RING * SLOT_BYTES + SMEM_W + CNN_CH * 4 + 64;
 constexpr int CONV_CTAS_PER_SM = 3;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -152,73 +157,115 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_but_last() {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+}
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<uint32_t*>(&h);
 }
 
-// Where tile t lies: its image, lattice row and first column.
-struct ConvTile {
+// A walk over tiles in strip order: image by image, 128-column strip by strip, row by row.
+struct Walk {
+    const CnnImage* img;
+    int nimg, im, tpr;   // tpr: strips of the image
     CnnImage I;
-    int y, x0;
-};
-__device__ __forceinline__ ConvTile conv_tile_of(const CnnImage* img, int nimg, int64_t tile) {
-    int im = 0;
-    while (im + 1 < nimg && img[im + 1].tile0 <= tile) ++im;
-    ConvTile t;
-    t.I = img[im];
-    const int64_t tloc = tile - t.I.tile0;
-    const int tpr = (t.I.W + CNN_TILE - 1) / CNN_TILE;  // tiles per row
-    t.y = (int)(tloc / tpr);
-    t.x0 = (int)(tloc % tpr) * CNN_TILE;
-    return t;
-}
-__device__ __forceinline__ ConvTile conv_tile(const CnnConvArgs& a, int64_t tile) {
-    return conv_tile_of(a.img, a.nimg, tile);
-}
-
-// Start the copies of a tile's halo into the planes at buf: [chunk][3][130] x 16
-// bytes, zero outside the image.  One commit group per call.
-__device__ __forceinline__ void conv_stage(const CnnConvArgs& a, const ConvTile& t, uint32_t buf,
-                                           int nch, int tid) {
-    const int nitem = nch * 3 * PLANE_COLS;
-    for (int i = tid; i < nitem; i += blockDim.x) {
-        const int c = i / (3 * PLANE_COLS);
-        const int rem = i - c * 3 * PLANE_COLS;
-        const int r = rem / PLANE_COLS;
-        const int col = rem - r * PLANE_COLS;
-        const int yy = t.y - 1 + r, xx = t.x0 - 1 + col;
-        const bool in = yy >= 0 && yy < t.I.H && xx >= 0 && xx < t.I.W;
-        const __nv_bfloat16* src = a.x;
-        if (in) src = a.x + (t.I.off + (int64_t)yy * t.I.W + xx) * a.cin + c * 8;
-        cp_async16(buf + c * PLANE_BYTES + (r * PLANE_COLS + col) * 16, src, in ? 16u : 0u);
+    int strip, y;
+    __device__ __forceinline__ void seek(const CnnImage* images, int n, int64_t tile) {
+        img = images;
+        nimg = n;
+        im = 0;
+        while (im + 1 < nimg && img[im + 1].tile0 <= tile) ++im;
+        I = img[im];
+        tpr = (I.W + CNN_TILE - 1) / CNN_TILE;
+        const int64_t t = tile - I.tile0;
+        strip = (int)(t / I.H);
+        y = (int)(t - (int64_t)strip * I.H);
     }
-    cp_async_commit();
-}
+    // To the next tile; true if it starts a new strip (nothing of its rows is there yet).
+    __device__ __forceinline__ bool next() {
+        if (++y < I.H) return false;
+        y = 0;
+        if (++strip == tpr) {
+            strip = 0;
+            if (im + 1 < nimg) {
+                I = img[++im];
+                tpr = (I.W + CNN_TILE - 1) / CNN_TILE;
+            }
+        }
+        return true;
+    }
+};
 
-// The 9 * Cin/16 MMAs of one tile: halo planes at in_addr, accumulator at tmem_d.
-__device__ __forceinline__ void conv_mma(uint32_t in_addr, uint32_t w_base, uint32_t tmem_d,
-                                         uint32_t idesc, int nch, int cout) {
-    uint32_t acc = 0;
-    for (int tap = 0; tap < 9; ++tap) {
-        const int dy = tap / 3, dx = tap % 3;  // 0..2 = offset + 1
-        for (int kc = 0; kc < nch / 2; ++kc) {
-            const uint32_t aaddr = in_addr + (2 * kc) * PLANE_BYTES + (dy * PLANE_COLS + dx) * 16;
-            const uint32_t baddr = w_base + (tap * nch + 2 * kc) * cout * 16;
-            umma_bf16(tmem_d, umma_desc(aaddr, PLANE_BYTES, 128), umma_desc(baddr, cout * 16, 128),
-                      idesc, acc);
-            acc = 1;
+// The rows that a range of tiles needs, in order: three for the first tile of a strip, one for
+// each further tile.  Row number n of this sequence lives in ring slot n % RING.
+struct RowStream {
+    Walk w;              // the tile whose rows come next
+    int64_t tiles;       // tiles left
+    int pend;            // rows left to fetch for it (the last is y + 1)
+    int count;           // rows fetched
+    __device__ __forceinline__ void init(const CnnImage* img, int nimg, int64_t t0, int64_t t1) {
+        tiles = t1 - t0;
+        if (tiles > 0) w.seek(img, nimg, t0);
+        pend = 3;
+        count = 0;
+    }
+    // Start the copies of the next row; with mirror, rows in the ring's first two slots are also
+    // written behind its end, so that three rows from any slot on lie in a line.
+    template <bool MIRROR>
+    __device__ __forceinline__ void fetch(const __nv_bfloat16* x, int cin, uint32_t ring, int tid) {
+        const int yy = w.y + 2 - pend, x0 = w.strip * CNN_TILE - 1;
+        const int slot = count % RING;
+        const bool row_in = yy >= 0 && yy < w.I.H;
+        const __nv_bfloat16* src = x + (w.I.off + (int64_t)(row_in ? yy : 0) * w.I.W) * cin;
+        const uint32_t dst = ring + slot * SLOT_BYTES;
+        const int sh = cin == 32 ? 2 : 1, nch = 1 << sh;
+        for (int i = tid; i < nch * PLANE_COLS; i += 128) {
+            const int c = i & (nch - 1), col = i >> sh, xx = x0 + col;
+            const bool in = row_in && xx >= 0 && xx < w.I.W;
+            const __nv_bfloat16* q = src + (in ? (int64_t)xx * cin + c * 8 : 0);
+            const uint32_t d = dst + c * PLANE_BYTES + col * 16;
+            cp_async16(d, q, in ? 16u : 0u);
+            if (MIRROR && slot < 2) cp_async16(d + RING * SLOT_BYTES, q, in ? 16u : 0u);
+        }
+        ++count;
+        if (--pend == 0) {
+            --tiles;
+            pend = tiles > 0 && w.next() ? 3 : 1;
         }
     }
+};
+
+// The 9 * Cin/16 MMAs of one tile whose first row is number `row` of the sequence.
+__device__ __forceinline__ void conv_mma(uint32_t ring, int row, uint32_t w_base, uint32_t tmem_d,
+                                         uint32_t idesc, int nch, int cout) {
+    uint32_t acc = 0;
+    for (int dy = 0; dy < 3; ++dy) {
+        const uint32_t slot = ring + ((row + dy) % RING) * SLOT_BYTES;
+        for (int dx = 0; dx < 3; ++dx)
+            for (int kc = 0; kc < nch / 2; ++kc) {
+                const uint32_t aaddr = slot + (2 * kc) * PLANE_BYTES + dx * 16;
+                const uint32_t baddr = w_base + ((dy * 3 + dx) * nch + 2 * kc) * cout * 16;
+                umma_bf16(tmem_d, umma_desc(aaddr, PLANE_BYTES, 128), umma_desc(baddr, cout * 16, 128), idesc,
+                          acc);
+                acc = 1;
+            }
+    }
+}
+
+__device__ __forceinline__ void st_global_32(void* p, const uint32_t* v) {
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                 "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
 }
 
 __global__ void __launch_bounds__(128) k_conv_tc(CnnConvArgs a) {
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t* s_w = smem + 2 * SMEM_IN;
-    uint64_t* s_bar = reinterpret_cast<uint64_t*>(smem + 2 * SMEM_IN + SMEM_W);  // [2]
-    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + 2 * SMEM_IN + SMEM_W + 16);
-    int* s_fail = reinterpret_cast<int*>(smem + 2 * SMEM_IN + SMEM_W + 20);
+    uint8_t* s_w = smem + RING * SLOT_BYTES;
+    float* s_bias = reinterpret_cast<float*>(s_w + SMEM_W);
+    uint64_t* s_bar = reinterpret_cast<uint64_t*>(s_w + SMEM_W + CNN_CH * 4);  // [2]
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(s_bar + 2);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cin = a.cin, cout = a.cout;
     const int nch = cin / 8;
@@ -232,18 +279,25 @@ __global__ void __launch_bounds__(128) k_conv_tc(CnnConvArgs a) {
     if (tid == 0) {
         mbar_init(s_bar, 1);
         mbar_init(s_bar + 1, 1);
-        *s_fail = 0;
+    }
+    // this CTA's tiles, a contiguous range
+    const int64_t t0 = a.ntiles * blockIdx.x / gridDim.x, t1 = a.ntiles * (blockIdx.x + 1) / gridDim.x;
+    const int64_t nt = t1 - t0;
+    const uint32_t ring = smem_u32(smem);
+    RowStream rows;
+    rows.init(a.img, a.nimg, t0, t1);
+    int c_prev = 0;  // rows fetched before the latest commit group
+    for (int h = 0; h < 2; ++h) {
+        c_prev = rows.count;
+        while (rows.tiles > 0 && rows.count < 3 * (h + 1)) rows.fetch<false>(a.x, cin, ring, tid);
+        cp_async_commit();
     }
     // weights, already in [tap][chunk][cout][8] order: one 16-byte copy per thread step
     const int wbytes = 9 * nch * cout * 16;
     for (int i = tid; i < wbytes / 16; i += blockDim.x)
         reinterpret_cast<uint4*>(s_w)[i] = reinterpret_cast<const uint4*>(a.wpack)[i];
-    // this CTA's tiles: blockIdx.x + k gridDim.x, k < nt
-    const int64_t nt = blockIdx.x < a.ntiles ? (a.ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    const uint32_t in_base = smem_u32(smem);
-    if (nt > 0) conv_stage(a, conv_tile(a, blockIdx.x), in_base, nch, tid);
-    if (nt > 1) conv_stage(a, conv_tile(a, blockIdx.x + gridDim.x), in_base + SMEM_IN, nch, tid);
-    cp_async_wait_all();  // tile 0's halo (tile 1's may still be in flight with it; both wait)
+    if (tid < cout) s_bias[tid] = a.bias ? a.bias[tid] : 0.0f;
+    cp_async_wait_but_last();  // the first tile's rows
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
     __syncthreads();
@@ -253,14 +307,32 @@ __global__ void __launch_bounds__(128) k_conv_tc(CnnConvArgs a) {
     const uint32_t w_base = smem_u32(s_w);
     uint32_t phase = 0u;  // bit b: parity of accumulator b's next completion
     int issued = 0;       // bit b: a committed MMA group on accumulator b not yet waited for
-    if (nt > 0 && tid == 0) {
-        conv_mma(in_base, w_base, tmem, idesc, nch, cout);
-        umma_commit(s_bar);
+    int row = 0;          // first row (number in the sequence) of the tile whose MMAs come next
+    Walk t;               // tile k
+    if (nt > 0) {
+        t.seek(a.img, a.nimg, t0);
+        if (tid == 0) {
+            conv_mma(ring, row, w_base, tmem, idesc, nch, cout);
+            umma_commit(s_bar);
+        }
+        issued = 1;
     }
-    if (nt > 0) issued = 1;
 
     for (int64_t k = 0; k < nt; ++k) {
         const int b = (int)(k & 1);
+        Walk tn = t;
+        const bool fresh = tn.next();
+        row += fresh ? 3 : 1;  // tile k + 1
+        const int x = t.strip * CNN_TILE + warp * 32 + lane;
+        const bool in = x < t.I.W;
+        const int64_t cell = t.I.off + (int64_t)t.y * t.I.W + x;
+        uint4 m[4];  // ReLU mask of tile k, on its way while the MMAs finish
+        if (a.epi == EPI_MASK_BF16 && in) {
+            const uint4* src = reinterpret_cast<const uint4*>(a.mask + cell * cout);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (q < cout / 8) m[q] = __ldg(src + q);
+        }
         // the MMAs of tile k
         const bool ok = mbar_wait_bounded(s_bar + b, (phase >> b) & 1u);
         if (ok) {
@@ -268,60 +340,55 @@ __global__ void __launch_bounds__(128) k_conv_tc(CnnConvArgs a) {
             issued &= ~(1 << b);
         } else {  // still in flight: the cleanup below waits for it again
             set_status(a.status, VIP_ERR_TIMEOUT);
-            *s_fail = 1;
         }
-        // tile k+1's halo (started two iterations ago, or in the prologue)
-        cp_async_wait_all();
+        // the rows of tile k + 1
+        if (row + 3 <= c_prev) cp_async_wait_but_last();
+        else cp_async_wait_all();
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_fence_before();
-        __syncthreads();
+        // (also: every warp has read accumulator 1 - b of tile k - 1)
+        const int failed = __syncthreads_or(!ok);
         tc_fence_after();
-        if (*s_fail) break;
+        if (failed) break;
         if (k + 1 < nt) {
             if (tid == 0) {
-                conv_mma(in_base + (1 - b) * SMEM_IN, w_base, tmem + (uint32_t)((1 - b) * 32), idesc,
-                         nch, cout);
+                conv_mma(ring, row, w_base, tmem + (uint32_t)((1 - b) * 32), idesc, nch, cout);
                 umma_commit(s_bar + (1 - b));
             }
             issued |= 1 << (1 - b);
         }
-        // tile k+2's halo into the buffer that tile k has released
-        if (k + 2 < nt)
-            conv_stage(a, conv_tile(a, blockIdx.x + (k + 2) * gridDim.x), in_base + b * SMEM_IN, nch, tid);
+        // rows into the slots that tile k has released
+        c_prev = rows.count;
+        while (rows.tiles > 0 && rows.count < row + RING) rows.fetch<false>(a.x, cin, ring, tid);
+        cp_async_commit();
         // epilogue of tile k: warp w reads TMEM lanes 32w..32w+31 = pixels x0 + 32w + lane
-        const ConvTile t = conv_tile(a, blockIdx.x + k * gridDim.x);
-        float v[32];
+        float v[32] = {};
         const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(b * 32);
         if (cout == 32) tmem_ld_x32(taddr, v);
         else tmem_ld_x16(taddr, v);
-        const int x = t.x0 + warp * 32 + lane;
-        if (x < t.I.W) {
-            const int64_t cell = t.I.off + (int64_t)t.y * t.I.W + x;
+        if (in) {
             if (a.epi == EPI_F32_CH0) {
-                a.y32[cell] = v[0] + (a.bias ? a.bias[0] : 0.0f);
+                a.y32[cell] = v[0] + s_bias[0];
             } else {
                 uint32_t packed[16];
-                for (int c2 = 0; c2 < cout / 2; ++c2) {
+#pragma unroll
+                for (int c2 = 0; c2 < 16; ++c2) {
                     float p0 = v[2 * c2], p1 = v[2 * c2 + 1];
                     if (a.epi == EPI_RELU_BF16) {
-                        p0 = fmaxf(p0 + a.bias[2 * c2], 0.0f);
-                        p1 = fmaxf(p1 + a.bias[2 * c2 + 1], 0.0f);
+                        p0 = fmaxf(p0 + s_bias[2 * c2], 0.0f);
+                        p1 = fmaxf(p1 + s_bias[2 * c2 + 1], 0.0f);
                     } else {  // gradient through the ReLU of the layer below
-                        const __nv_bfloat16* m = a.mask + cell * cout;
-                        p0 = __bfloat162float(m[2 * c2]) > 0.0f ? p0 : 0.0f;
-                        p1 = __bfloat162float(m[2 * c2 + 1]) > 0.0f ? p1 : 0.0f;
+                        const uint32_t mm = reinterpret_cast<const uint32_t*>(m)[c2];
+                        p0 = __uint_as_float(mm << 16) > 0.0f ? p0 : 0.0f;
+                        p1 = __uint_as_float(mm & 0xffff0000u) > 0.0f ? p1 : 0.0f;
                     }
                     packed[c2] = pack_bf16(p0, p1);
                 }
-                uint4* dst = reinterpret_cast<uint4*>(a.y + cell * cout);
-                for (int q = 0; q < cout / 8; ++q)
-                    dst[q] = make_uint4(packed[4 * q], packed[4 * q + 1], packed[4 * q + 2],
-                                        packed[4 * q + 3]);
+                st_global_32(a.y + cell * cout, packed);
+                if (cout == 32) st_global_32(a.y + cell * cout + 16, packed + 8);
             }
         }
-        // accumulator b is read out before the MMAs of tile k+2 overwrite it
-        tc_fence_before();
-        __syncthreads();
+        t = tn;
     }
     // after a failed wait MMAs may still be in flight: wait for every committed group
     // once more (bounded) before freeing TMEM; no copy is left in flight either
@@ -337,20 +404,27 @@ __global__ void __launch_bounds__(128) k_conv_tc(CnnConvArgs a) {
 }
 
 // Weight gradients dW[tap][ci][co] = sum_p x[p + off(tap)][ci] gy[p][co] as MMAs on the
-// tensor cores, K = pixels.  The halo is staged as for the convolution, channel-chunk
-// planar, here with four lattice rows: [row][chunk][col] x 16 bytes.  Read with the
-// pixel as K, an 8-pixel x 8-channel block (128 contiguous bytes) is a core matrix of
-// an MN-major operand, so A (M = 4 rows x 32 channels, the fourth row's products
-// discarded) and B (N = cout channels of gy, staged [chunk][pixel] x 16 bytes) need no
-// transpose, and the three column offsets of the taps are start addresses 16 bytes
-// apart.  Each block accumulates all its tiles in TMEM (three 32-column accumulators,
-// one per column offset) and writes one FP32 partial; the bias gradients are summed
-// on the side in pixel order.
-constexpr int WG_ROWS = 4;
-constexpr int WG_PLANE = PLANE_COLS * 16;                     // 2080: one row of one chunk
-constexpr int WG_SMEM_X = WG_ROWS * MAX_CHUNKS * WG_PLANE;    // 33280
+// tensor cores, K = pixels.  The input rows are staged as for the convolution, in a ring walked
+// down the strips.  Read with the pixel as K, an 8-pixel x 8-channel block (128 contiguous bytes)
+// is a core matrix of an MN-major operand, so A (M = 4 rows x 32 channels, a tile's three rows and
+// whatever lies in the slot behind them: its products are discarded) and B (N = cout channels of
+// gy, staged [chunk][pixel] x 16 bytes) need no transpose, and the three column offsets of the
+// taps are start addresses 16 bytes apart.  M runs over rows at one stride, so rows in the ring's
+// first two slots are written twice, the second time behind its end.  Each block accumulates all
+// its tiles in TMEM (three 32-column accumulators, one per column offset) and writes one FP32
+// partial.  The bias gradients are summed on the side: warp w takes gy's channels 8w..8w+7, each
+// lane four pixels of a tile, and the lanes add up once at the end.
+//
+// In iteration k the CTA issues tile k's MMAs, sums its biases, waits for the MMAs of tile k-1
+// and starts the copies of the rows and of gy (three buffers) that its release makes room for.
+// 32 channels at 513 x 1025: 43 us (the MMAs' reads of A alone 12; 93 when each tile waited
+// for the copies of four rows and for its MMAs in turn, and one thread per channel summed the
+// bias over 128 pixels).
+constexpr int WG_SLOTS = RING + 3;
+constexpr int WG_SMEM_X = WG_SLOTS * SLOT_BYTES;              // 74880
 constexpr int WG_SMEM_G = MAX_CHUNKS * CNN_TILE * 16;         // 8192
-constexpr int SMEM_WGRAD = WG_SMEM_X + WG_SMEM_G + 64;
+constexpr int WG_GBUF = 3;
+constexpr int SMEM_WGRAD = WG_SMEM_X + WG_GBUF * WG_SMEM_G + 64;   // two CTAs per SM
 // MN-major core matrices, no swizzle: the descriptor's leading-dimension offset is
 // the byte distance between core matrices adjacent along K (8 more pixels: 128 bytes
 // in both staged layouts), the stride-dimension offset the distance along M/N (8 more
@@ -362,16 +436,25 @@ __host__ __device__ constexpr uint32_t umma_idesc_mn(int M, int N) {
     return umma_idesc(M, N) | (1u << 15) | (1u << 16);  // A and B MN-major
 }
 
+// gy of a tile's 128 pixels, zero beyond the row
+__device__ __forceinline__ void wgrad_fetch_gy(const __nv_bfloat16* gy, const Walk& t, int cout, uint32_t buf,
+                                               int tid) {
+    const int sh = cout == 32 ? 2 : 1, nch = 1 << sh, x0 = t.strip * CNN_TILE;
+    const __nv_bfloat16* src = gy + (t.I.off + (int64_t)t.y * t.I.W) * cout;
+    for (int i = tid; i < nch * CNN_TILE; i += 128) {
+        const int c = i & (nch - 1), p = i >> sh;
+        const bool in = x0 + p < t.I.W;
+        cp_async16(buf + (c * CNN_TILE + p) * 16, src + (in ? (int64_t)(x0 + p) * cout + c * 8 : 0), in ? 16u : 0u);
+    }
+}
+
 __global__ void __launch_bounds__(128) k_wgrad_tc(CnnWgradArgs a) {
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t* s_x = smem;
     uint8_t* s_g = smem + WG_SMEM_X;
-    uint64_t* s_bar = reinterpret_cast<uint64_t*>(smem + WG_SMEM_X + WG_SMEM_G);
-    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(smem + WG_SMEM_X + WG_SMEM_G + 8);
-    int* s_fail = reinterpret_cast<int*>(smem + WG_SMEM_X + WG_SMEM_G + 12);
+    uint64_t* s_bar = reinterpret_cast<uint64_t*>(s_g + WG_GBUF * WG_SMEM_G);   // [2]
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(s_bar + 2);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cin = a.cin, cout = a.cout;
-    const int nch = cin / 8, nchg = cout / 8;
     const int ncol = 128;  // three accumulators of 32 columns
 
     if (warp == 0) {
@@ -381,97 +464,125 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(CnnWgradArgs a) {
     }
     if (tid == 0) {
         mbar_init(s_bar, 1);
-        *s_fail = 0;
+        mbar_init(s_bar + 1, 1);
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
     const uint32_t idesc = umma_idesc_mn(128, cout);
-    const uint32_t xb = smem_u32(s_x), gb = smem_u32(s_g);
-    const uint32_t lbo = WG_K_STRIDE, sbo_a = WG_PLANE, sbo_b = CNN_TILE * 16;
-    uint32_t phase = 0u;
-    bool pending = false;
-    float bacc = 0.0f;
-    const int64_t nt = blockIdx.x < a.ntiles ? (a.ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    for (int64_t k = 0; k < nt; ++k) {
-        const ConvTile t = conv_tile_of(a.img, a.nimg, blockIdx.x + k * gridDim.x);
-        // rows y-1 .. y+2 of the input, columns x0-1 .. x0+128, zero outside the image
-        const int nx_items = WG_ROWS * nch * PLANE_COLS;
-        for (int i = tid; i < nx_items; i += blockDim.x) {
-            const int r = i / (nch * PLANE_COLS);
-            const int rem = i - r * nch * PLANE_COLS;
-            const int c = rem / PLANE_COLS;
-            const int col = rem - c * PLANE_COLS;
-            const int yy = t.y - 1 + r, xx = t.x0 - 1 + col;
-            const bool in = yy >= 0 && yy < t.I.H && xx >= 0 && xx < t.I.W;
-            const __nv_bfloat16* src = a.x;
-            if (in) src = a.x + (t.I.off + (int64_t)yy * t.I.W + xx) * cin + c * 8;
-            cp_async16(xb + (r * MAX_CHUNKS + c) * WG_PLANE + col * 16, src, in ? 16u : 0u);
-        }
-        // gy of the tile's 128 pixels, zero beyond the row
-        for (int i = tid; i < nchg * CNN_TILE; i += blockDim.x) {
-            const int c = i / CNN_TILE, p = i - c * CNN_TILE;
-            const int xx = t.x0 + p;
-            const bool in = xx < t.I.W;
-            const __nv_bfloat16* src = a.gy;
-            if (in) src = a.gy + (t.I.off + (int64_t)t.y * t.I.W + xx) * cout + c * 8;
-            cp_async16(gb + (c * CNN_TILE + p) * 16, src, in ? 16u : 0u);
+    const uint32_t xb = smem_u32(smem), gb = smem_u32(s_g);
+    const uint32_t lbo = WG_K_STRIDE, sbo_a = PLANE_BYTES, sbo_b = CNN_TILE * 16;
+    const int64_t t0 = a.ntiles * blockIdx.x / gridDim.x, t1 = a.ntiles * (blockIdx.x + 1) / gridDim.x;
+    const int64_t nt = t1 - t0;
+    RowStream rows;
+    rows.init(a.img, a.nimg, t0, t1);
+    Walk t, tg;              // tile k; the tile whose gy comes next
+    int64_t gleft = nt;      // tiles whose gy is still to fetch
+    if (nt > 0) {
+        t.seek(a.img, a.nimg, t0);
+        tg = t;
+    }
+    int c_prev = 0;
+    for (int h = 0; h < 2; ++h) {
+        c_prev = rows.count;
+        while (rows.tiles > 0 && rows.count < 3 * (h + 1)) rows.fetch<true>(a.x, cin, xb, tid);
+        if (gleft > 0) {
+            wgrad_fetch_gy(a.gy, tg, cout, gb + h * WG_SMEM_G, tid);
+            if (--gleft > 0) tg.next();
         }
         cp_async_commit();
-        cp_async_wait_all();
+    }
+    float bacc[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) bacc[j] = 0.0f;
+    int64_t issued = 0, waited = 0;   // tiles whose MMAs were committed, and waited for
+    bool ok = true;
+    int failed = 0;
+    int row = 0, gbuf = 0;
+    for (int64_t k = 0; k < nt; ++k) {
+        if (row + 3 <= c_prev) cp_async_wait_but_last();
+        else cp_async_wait_all();
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_fence_before();
-        __syncthreads();
+        failed = __syncthreads_or(!ok);
         tc_fence_after();
-        if (tid < cout) {  // bias gradient, pixel order
-            const __nv_bfloat16* g = reinterpret_cast<const __nv_bfloat16*>(s_g) + (tid >> 3) * CNN_TILE * 8 + (tid & 7);
-            for (int p = 0; p < CNN_TILE; ++p) bacc += __bfloat162float(g[p * 8]);
-        }
+        if (failed) break;
         if (tid == 0) {
+            const uint32_t ab = xb + (row % RING) * SLOT_BYTES, bb = gb + gbuf * WG_SMEM_G;
             for (int dx = 0; dx < 3; ++dx)
-                for (int kc = 0; kc < CNN_TILE / 16; ++kc) {
-                    const uint32_t aaddr = xb + dx * 16 + kc * 2 * WG_K_STRIDE;
-                    const uint32_t baddr = gb + kc * 2 * WG_K_STRIDE;
-                    umma_bf16(tmem + (uint32_t)(dx * 32), umma_desc(aaddr, lbo, sbo_a),
-                              umma_desc(baddr, lbo, sbo_b), idesc, (k > 0 || kc > 0) ? 1u : 0u);
+                for (int kc = 0; kc < CNN_TILE / 16; ++kc)
+                    umma_bf16(tmem + (uint32_t)(dx * 32), umma_desc(ab + dx * 16 + kc * 2 * WG_K_STRIDE, lbo, sbo_a),
+                              umma_desc(bb + kc * 2 * WG_K_STRIDE, lbo, sbo_b), idesc, (k > 0 || kc > 0) ? 1u : 0u);
+            umma_commit(s_bar + (k & 1));
+        }
+        ++issued;
+        if (warp < cout / 8) {  // bias gradient
+            const uint4* g = reinterpret_cast<const uint4*>(s_g + gbuf * WG_SMEM_G) + warp * CNN_TILE + lane;
+#pragma unroll
+            for (int q = 0; q < CNN_TILE / 32; ++q) {
+                const uint4 v = g[q * 32];
+                const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    bacc[2 * j] += __uint_as_float(u[j] << 16);
+                    bacc[2 * j + 1] += __uint_as_float(u[j] & 0xffff0000u);
                 }
-            umma_commit(s_bar);
+            }
         }
-        pending = true;
-        const bool ok = mbar_wait_bounded(s_bar, phase);
+        if (k > 0) {  // the MMAs of tile k - 1
+            ok = mbar_wait_bounded(s_bar + ((k - 1) & 1), (uint32_t)((k - 1) >> 1) & 1u);
+            if (ok) ++waited;
+            else set_status(a.status, VIP_ERR_TIMEOUT);
+        }
+        c_prev = rows.count;
         if (ok) {
-            phase ^= 1u;
-            pending = false;
-        } else {
-            set_status(a.status, VIP_ERR_TIMEOUT);
-            *s_fail = 1;
+            while (rows.tiles > 0 && rows.count < row + RING) rows.fetch<true>(a.x, cin, xb, tid);
+            if (gleft > 0) {
+                wgrad_fetch_gy(a.gy, tg, cout, gb + (gbuf == 0 ? 2 : gbuf - 1) * WG_SMEM_G, tid);  // tile k + 2
+                if (--gleft > 0) tg.next();
+            }
         }
-        tc_fence_before();
-        __syncthreads();  // the buffers are restaged by the next tile
-        tc_fence_after();
-        if (*s_fail) break;
+        cp_async_commit();
+        row += t.next() ? 3 : 1;
+        gbuf = gbuf == WG_GBUF - 1 ? 0 : gbuf + 1;
     }
+    // the last tile's MMAs (after a failed wait, all that may still be in flight)
+    for (; waited < issued; ++waited)
+        if (!mbar_wait_bounded(s_bar + (waited & 1), (uint32_t)(waited >> 1) & 1u)) {
+            set_status(a.status, VIP_ERR_TIMEOUT);
+            ok = false;
+        }
+    cp_async_wait_all();
+    tc_fence_before();
+    failed |= __syncthreads_or(!ok);
+    tc_fence_after();
     const int nent = 9 * cin * cout;
     float* dst = a.part + (int64_t)blockIdx.x * (nent + cout);
-    if (nt > 0 && !*s_fail) {
-        // warp w holds TMEM lanes 32w..32w+31 = row w of the halo (tap row dy = w), channel = lane
+    if (nt > 0 && !failed) {
+        // warp w holds TMEM lanes 32w..32w+31 = row w of the window (tap row dy = w), channel = lane
         for (int dx = 0; dx < 3; ++dx) {
             float v[32];
             const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(dx * 32);
             if (cout == 32) tmem_ld_x32(taddr, v);
             else tmem_ld_x16(taddr, v);
             if (warp < 3 && lane < cin) {
-                float* o = dst + ((int64_t)(warp * 3 + dx) * cin + lane) * cout;
-                for (int co = 0; co < cout; ++co) o[co] = v[co];
+                float4* o = reinterpret_cast<float4*>(dst + ((int64_t)(warp * 3 + dx) * cin + lane) * cout);
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    if (q < cout / 4) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
             }
         }
     } else {
         for (int e = tid; e < nent; e += blockDim.x) dst[e] = 0.0f;
     }
-    if (tid < cout) dst[nent + tid] = bacc;
-    cp_async_wait_all();
-    if (tid == 0 && pending) mbar_wait_bounded(s_bar, phase);
+    if (warp < cout / 8)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            float v = bacc[j];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) dst[nent + warp * 8 + j] = v;
+        }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
