@@ -356,6 +356,7 @@ __global__ void __launch_bounds__(256) k_wgrad_sum(const float* __restrict__ par
     const int nent = 9 * cin * cout, e = blockIdx.x * 32 + lane;
     double s = 0.0;
     if (e < nent + cout)
+#pragma unroll 8
         for (int b = warp; b < nblocks; b += 8) s += part[(int64_t)b * (nent + cout) + e];
     s_sum[warp][lane] = s;
     __syncthreads();

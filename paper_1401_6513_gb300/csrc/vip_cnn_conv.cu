@@ -20,9 +20,10 @@
 // freed.
 //
 // A layer of 32 channels moves 67 MB at 513 x 1025 (10 us) and its MMAs read 4 KB of A each from
-// shared memory (9 us).  It takes 35 to 41 us; 98 when every tile fetched its three rows with copies
-// that touched one chunk of 32 pixels at a time, wrote 16 bytes at a time and read the ReLU mask
-// element by element.
+// shared memory (9 us).  It takes 33 us, bound by the instructions and waits of 12 warps per
+// SM (35 to 41 with the channel counts as run-time numbers; 98 when every tile fetched its three
+// rows with copies that touched one chunk of 32 pixels at a time, wrote 16 bytes at a time and
+// read the ReLU mask element by element).
 #include <algorithm>
 #include <cstdio>
 
@@ -89,6 +90,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 
 // Bounded wait for the phase with the given parity; false after 2 s.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity) {
+    if (mbar_try_wait(bar, parity)) return true;
     uint64_t t0 = gtime();
     while (!mbar_try_wait(bar, parity)) {
         if (gtime() - t0 > 2000000000ull) return false;
@@ -205,30 +207,34 @@ struct RowStream {
     int64_t tiles;       // tiles left
     int pend;            // rows left to fetch for it (the last is y + 1)
     int count;           // rows fetched
+    int slot;            // count % RING
     __device__ __forceinline__ void init(const CnnImage* img, int nimg, int64_t t0, int64_t t1) {
         tiles = t1 - t0;
         if (tiles > 0) w.seek(img, nimg, t0);
         pend = 3;
         count = 0;
+        slot = 0;
     }
     // Start the copies of the next row; with mirror, rows in the ring's first two slots are also
     // written behind its end, so that three rows from any slot on lie in a line.
-    template <bool MIRROR>
-    __device__ __forceinline__ void fetch(const __nv_bfloat16* x, int cin, uint32_t ring, int tid) {
-        const int yy = w.y + 2 - pend, x0 = w.strip * CNN_TILE - 1;
-        const int slot = count % RING;
+    template <int CIN, bool MIRROR>
+    __device__ __forceinline__ void fetch(const __nv_bfloat16* x, uint32_t ring, int tid) {
+        constexpr int NCH = CIN / 8, PIX = 128 / NCH;   // chunks of a pixel; pixels per pass of 128 threads
+        const int yy = w.y + 2 - pend;
         const bool row_in = yy >= 0 && yy < w.I.H;
-        const __nv_bfloat16* src = x + (w.I.off + (int64_t)(row_in ? yy : 0) * w.I.W) * cin;
-        const uint32_t dst = ring + slot * SLOT_BYTES;
-        const int sh = cin == 32 ? 2 : 1, nch = 1 << sh;
-        for (int i = tid; i < nch * PLANE_COLS; i += 128) {
-            const int c = i & (nch - 1), col = i >> sh, xx = x0 + col;
-            const bool in = row_in && xx >= 0 && xx < w.I.W;
-            const __nv_bfloat16* q = src + (in ? (int64_t)xx * cin + c * 8 : 0);
-            const uint32_t d = dst + c * PLANE_BYTES + col * 16;
-            cp_async16(d, q, in ? 16u : 0u);
-            if (MIRROR && slot < 2) cp_async16(d + RING * SLOT_BYTES, q, in ? 16u : 0u);
+        const int c = tid % NCH, col0 = tid / NCH, xx = w.strip * CNN_TILE - 1 + col0;
+        const __nv_bfloat16* src = x + (w.I.off + (int64_t)(row_in ? yy : 0) * w.I.W) * CIN;
+        const uint32_t d = ring + slot * SLOT_BYTES + c * PLANE_BYTES + col0 * 16;
+#pragma unroll
+        for (int j = 0; j < (PLANE_COLS + PIX - 1) / PIX; ++j) {
+            if (j * PIX + PIX > PLANE_COLS && j * PIX + col0 >= PLANE_COLS) break;
+            const int xj = xx + j * PIX;
+            const bool in = row_in && xj >= 0 && xj < w.I.W;
+            const __nv_bfloat16* q = in ? src + (int64_t)xj * CIN + c * 8 : x;
+            cp_async16(d + j * PIX * 16, q, in ? 16u : 0u);
+            if (MIRROR && slot < 2) cp_async16(d + RING * SLOT_BYTES + j * PIX * 16, q, in ? 16u : 0u);
         }
+        slot = slot == RING - 1 ? 0 : slot + 1;
         ++count;
         if (--pend == 0) {
             --tiles;
@@ -237,20 +243,23 @@ struct RowStream {
     }
 };
 
-// The 9 * Cin/16 MMAs of one tile whose first row is number `row` of the sequence.
-__device__ __forceinline__ void conv_mma(uint32_t ring, int row, uint32_t w_base, uint32_t tmem_d,
-                                         uint32_t idesc, int nch, int cout) {
-    uint32_t acc = 0;
+// The 9 * Cin/16 MMAs of one tile whose first row lies in slot `slot`.  Descriptors differ in
+// their start address only (bits 0 to 13, in units of 16 bytes).
+template <int CIN, int COUT>
+__device__ __forceinline__ void conv_mma(uint32_t ring, int slot, uint32_t w_base, uint32_t tmem_d) {
+    constexpr int NCH = CIN / 8;
+    constexpr uint32_t idesc = umma_idesc(CNN_TILE, COUT);
+    const uint64_t bd = umma_desc(w_base, COUT * 16, 128);
+#pragma unroll
     for (int dy = 0; dy < 3; ++dy) {
-        const uint32_t slot = ring + ((row + dy) % RING) * SLOT_BYTES;
+        const uint64_t ad = umma_desc(ring + slot * SLOT_BYTES, PLANE_BYTES, 128);
+        slot = slot == RING - 1 ? 0 : slot + 1;
+#pragma unroll
         for (int dx = 0; dx < 3; ++dx)
-            for (int kc = 0; kc < nch / 2; ++kc) {
-                const uint32_t aaddr = slot + (2 * kc) * PLANE_BYTES + dx * 16;
-                const uint32_t baddr = w_base + ((dy * 3 + dx) * nch + 2 * kc) * cout * 16;
-                umma_bf16(tmem_d, umma_desc(aaddr, PLANE_BYTES, 128), umma_desc(baddr, cout * 16, 128), idesc,
-                          acc);
-                acc = 1;
-            }
+#pragma unroll
+            for (int kc = 0; kc < NCH / 2; ++kc)
+                umma_bf16(tmem_d, ad + (2 * kc * PLANE_BYTES + dx * 16) / 16,
+                          bd + ((dy * 3 + dx) * NCH + 2 * kc) * COUT, idesc, dy + dx + kc > 0 ? 1u : 0u);
     }
 }
 
@@ -260,6 +269,7 @@ __device__ __forceinline__ void st_global_32(void* p, const uint32_t* v) {
                  : "memory");
 }
 
+template <int CIN, int COUT, int EPI>
 __global__ void __launch_bounds__(128) k_conv_tc(CnnConvArgs a) {
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* s_w = smem + RING * SLOT_BYTES;
@@ -267,8 +277,6 @@ __global__ void __launch_bounds__(128) k_conv_tc(CnnConvArgs a) {
     uint64_t* s_bar = reinterpret_cast<uint64_t*>(s_w + SMEM_W + CNN_CH * 4);  // [2]
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(s_bar + 2);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int cin = a.cin, cout = a.cout;
-    const int nch = cin / 8;
     const int ncol = 64;  // TMEM columns: two accumulators of 32 (>= cout) columns
 
     if (warp == 0) {
@@ -289,30 +297,28 @@ __global__ void __launch_bounds__(128) k_conv_tc(CnnConvArgs a) {
     int c_prev = 0;  // rows fetched before the latest commit group
     for (int h = 0; h < 2; ++h) {
         c_prev = rows.count;
-        while (rows.tiles > 0 && rows.count < 3 * (h + 1)) rows.fetch<false>(a.x, cin, ring, tid);
+        while (rows.tiles > 0 && rows.count < 3 * (h + 1)) rows.fetch<CIN, false>(a.x, ring, tid);
         cp_async_commit();
     }
     // weights, already in [tap][chunk][cout][8] order: one 16-byte copy per thread step
-    const int wbytes = 9 * nch * cout * 16;
-    for (int i = tid; i < wbytes / 16; i += blockDim.x)
+    for (int i = tid; i < 9 * CIN / 8 * COUT; i += 128)
         reinterpret_cast<uint4*>(s_w)[i] = reinterpret_cast<const uint4*>(a.wpack)[i];
-    if (tid < cout) s_bias[tid] = a.bias ? a.bias[tid] : 0.0f;
+    if (tid < COUT) s_bias[tid] = a.bias ? a.bias[tid] : 0.0f;
     cp_async_wait_but_last();  // the first tile's rows
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
-    const uint32_t idesc = umma_idesc(CNN_TILE, cout);
     const uint32_t w_base = smem_u32(s_w);
     uint32_t phase = 0u;  // bit b: parity of accumulator b's next completion
     int issued = 0;       // bit b: a committed MMA group on accumulator b not yet waited for
-    int row = 0;          // first row (number in the sequence) of the tile whose MMAs come next
+    int row = 0, slot = 0;  // first row (number in the sequence) of the tile whose MMAs come next, its slot
     Walk t;               // tile k
     if (nt > 0) {
         t.seek(a.img, a.nimg, t0);
         if (tid == 0) {
-            conv_mma(ring, row, w_base, tmem, idesc, nch, cout);
+            conv_mma<CIN, COUT>(ring, 0, w_base, tmem);
             umma_commit(s_bar);
         }
         issued = 1;
@@ -321,17 +327,17 @@ __global__ void __launch_bounds__(128) k_conv_tc(CnnConvArgs a) {
     for (int64_t k = 0; k < nt; ++k) {
         const int b = (int)(k & 1);
         Walk tn = t;
-        const bool fresh = tn.next();
-        row += fresh ? 3 : 1;  // tile k + 1
+        const int step = tn.next() ? 3 : 1;
+        row += step;  // tile k + 1
+        slot = slot + step >= RING ? slot + step - RING : slot + step;
         const int x = t.strip * CNN_TILE + warp * 32 + lane;
         const bool in = x < t.I.W;
         const int64_t cell = t.I.off + (int64_t)t.y * t.I.W + x;
-        uint4 m[4];  // ReLU mask of tile k, on its way while the MMAs finish
-        if (a.epi == EPI_MASK_BF16 && in) {
-            const uint4* src = reinterpret_cast<const uint4*>(a.mask + cell * cout);
+        uint4 m[COUT / 8];  // ReLU mask of tile k, on its way while the MMAs finish
+        if (EPI == EPI_MASK_BF16 && in) {
+            const uint4* src = reinterpret_cast<const uint4*>(a.mask + cell * COUT);
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (q < cout / 8) m[q] = __ldg(src + q);
+            for (int q = 0; q < COUT / 8; ++q) m[q] = __ldg(src + q);
         }
         // the MMAs of tile k
         const bool ok = mbar_wait_bounded(s_bar + b, (phase >> b) & 1u);
@@ -352,40 +358,46 @@ __global__ void __launch_bounds__(128) k_conv_tc(CnnConvArgs a) {
         if (failed) break;
         if (k + 1 < nt) {
             if (tid == 0) {
-                conv_mma(ring, row, w_base, tmem + (uint32_t)((1 - b) * 32), idesc, nch, cout);
+                conv_mma<CIN, COUT>(ring, slot, w_base, tmem + (uint32_t)((1 - b) * 32));
                 umma_commit(s_bar + (1 - b));
             }
             issued |= 1 << (1 - b);
         }
         // rows into the slots that tile k has released
         c_prev = rows.count;
-        while (rows.tiles > 0 && rows.count < row + RING) rows.fetch<false>(a.x, cin, ring, tid);
+        while (rows.tiles > 0 && rows.count < row + RING) rows.fetch<CIN, false>(a.x, ring, tid);
         cp_async_commit();
         // epilogue of tile k: warp w reads TMEM lanes 32w..32w+31 = pixels x0 + 32w + lane
-        float v[32] = {};
+        float v[COUT];
         const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(b * 32);
-        if (cout == 32) tmem_ld_x32(taddr, v);
+        if constexpr (COUT == 32) tmem_ld_x32(taddr, v);
         else tmem_ld_x16(taddr, v);
         if (in) {
-            if (a.epi == EPI_F32_CH0) {
+            if constexpr (EPI == EPI_F32_CH0) {
                 a.y32[cell] = v[0] + s_bias[0];
             } else {
-                uint32_t packed[16];
+                uint32_t packed[COUT / 2];
 #pragma unroll
-                for (int c2 = 0; c2 < 16; ++c2) {
-                    float p0 = v[2 * c2], p1 = v[2 * c2 + 1];
-                    if (a.epi == EPI_RELU_BF16) {
-                        p0 = fmaxf(p0 + s_bias[2 * c2], 0.0f);
-                        p1 = fmaxf(p1 + s_bias[2 * c2 + 1], 0.0f);
+                for (int q = 0; q < COUT / 4; ++q) {
+                    float* p = v + 4 * q;
+                    if constexpr (EPI == EPI_RELU_BF16) {
+                        const float4 bq = reinterpret_cast<const float4*>(s_bias)[q];
+                        p[0] = fmaxf(p[0] + bq.x, 0.0f);
+                        p[1] = fmaxf(p[1] + bq.y, 0.0f);
+                        p[2] = fmaxf(p[2] + bq.z, 0.0f);
+                        p[3] = fmaxf(p[3] + bq.w, 0.0f);
                     } else {  // gradient through the ReLU of the layer below
-                        const uint32_t mm = reinterpret_cast<const uint32_t*>(m)[c2];
-                        p0 = __uint_as_float(mm << 16) > 0.0f ? p0 : 0.0f;
-                        p1 = __uint_as_float(mm & 0xffff0000u) > 0.0f ? p1 : 0.0f;
+                        const uint32_t m0 = q & 1 ? m[q / 2].z : m[q / 2].x, m1 = q & 1 ? m[q / 2].w : m[q / 2].y;
+                        p[0] = __uint_as_float(m0 << 16) > 0.0f ? p[0] : 0.0f;
+                        p[1] = __uint_as_float(m0 & 0xffff0000u) > 0.0f ? p[1] : 0.0f;
+                        p[2] = __uint_as_float(m1 << 16) > 0.0f ? p[2] : 0.0f;
+                        p[3] = __uint_as_float(m1 & 0xffff0000u) > 0.0f ? p[3] : 0.0f;
                     }
-                    packed[c2] = pack_bf16(p0, p1);
+                    packed[2 * q] = pack_bf16(p[0], p[1]);
+                    packed[2 * q + 1] = pack_bf16(p[2], p[3]);
                 }
-                st_global_32(a.y + cell * cout, packed);
-                if (cout == 32) st_global_32(a.y + cell * cout + 16, packed + 8);
+#pragma unroll
+                for (int q = 0; q < COUT / 16; ++q) st_global_32(a.y + cell * COUT + 16 * q, packed + 8 * q);
             }
         }
         t = tn;
@@ -417,7 +429,7 @@ __global__ void __launch_bounds__(128) k_conv_tc(CnnConvArgs a) {
 //
 // In iteration k the CTA issues tile k's MMAs, sums its biases, waits for the MMAs of tile k-1
 // and starts the copies of the rows and of gy (three buffers) that its release makes room for.
-// 32 channels at 513 x 1025: 43 us (the MMAs' reads of A alone 12; 93 when each tile waited
+// 32 channels at 513 x 1025: 40 us (the MMAs' reads of A alone 12; 93 when each tile waited
 // for the copies of four rows and for its MMAs in turn, and one thread per channel summed the
 // bias over 128 pixels).
 constexpr int WG_SLOTS = RING + 3;
@@ -437,24 +449,26 @@ __host__ __device__ constexpr uint32_t umma_idesc_mn(int M, int N) {
 }
 
 // gy of a tile's 128 pixels, zero beyond the row
-__device__ __forceinline__ void wgrad_fetch_gy(const __nv_bfloat16* gy, const Walk& t, int cout, uint32_t buf,
-                                               int tid) {
-    const int sh = cout == 32 ? 2 : 1, nch = 1 << sh, x0 = t.strip * CNN_TILE;
-    const __nv_bfloat16* src = gy + (t.I.off + (int64_t)t.y * t.I.W) * cout;
-    for (int i = tid; i < nch * CNN_TILE; i += 128) {
-        const int c = i & (nch - 1), p = i >> sh;
-        const bool in = x0 + p < t.I.W;
-        cp_async16(buf + (c * CNN_TILE + p) * 16, src + (in ? (int64_t)(x0 + p) * cout + c * 8 : 0), in ? 16u : 0u);
+template <int COUT>
+__device__ __forceinline__ void wgrad_fetch_gy(const __nv_bfloat16* gy, const Walk& t, uint32_t buf, int tid) {
+    constexpr int NCH = COUT / 8, PIX = 128 / NCH;
+    const int c = tid % NCH, p0 = tid / NCH, x0 = t.strip * CNN_TILE + p0;
+    const __nv_bfloat16* src = gy + (t.I.off + (int64_t)t.y * t.I.W + x0) * COUT + c * 8;
+    const uint32_t d = buf + (c * CNN_TILE + p0) * 16;
+#pragma unroll
+    for (int j = 0; j < CNN_TILE / PIX; ++j) {
+        const bool in = x0 + j * PIX < t.I.W;
+        cp_async16(d + j * PIX * 16, in ? src + j * PIX * COUT : gy, in ? 16u : 0u);
     }
 }
 
+template <int CIN, int COUT>
 __global__ void __launch_bounds__(128) k_wgrad_tc(CnnWgradArgs a) {
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* s_g = smem + WG_SMEM_X;
     uint64_t* s_bar = reinterpret_cast<uint64_t*>(s_g + WG_GBUF * WG_SMEM_G);   // [2]
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(s_bar + 2);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int cin = a.cin, cout = a.cout;
     const int ncol = 128;  // three accumulators of 32 columns
 
     if (warp == 0) {
@@ -470,7 +484,7 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(CnnWgradArgs a) {
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
-    const uint32_t idesc = umma_idesc_mn(128, cout);
+    const uint32_t idesc = umma_idesc_mn(128, COUT);
     const uint32_t xb = smem_u32(smem), gb = smem_u32(s_g);
     const uint32_t lbo = WG_K_STRIDE, sbo_a = PLANE_BYTES, sbo_b = CNN_TILE * 16;
     const int64_t t0 = a.ntiles * blockIdx.x / gridDim.x, t1 = a.ntiles * (blockIdx.x + 1) / gridDim.x;
@@ -486,9 +500,9 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(CnnWgradArgs a) {
     int c_prev = 0;
     for (int h = 0; h < 2; ++h) {
         c_prev = rows.count;
-        while (rows.tiles > 0 && rows.count < 3 * (h + 1)) rows.fetch<true>(a.x, cin, xb, tid);
+        while (rows.tiles > 0 && rows.count < 3 * (h + 1)) rows.fetch<CIN, true>(a.x, xb, tid);
         if (gleft > 0) {
-            wgrad_fetch_gy(a.gy, tg, cout, gb + h * WG_SMEM_G, tid);
+            wgrad_fetch_gy<COUT>(a.gy, tg, gb + h * WG_SMEM_G, tid);
             if (--gleft > 0) tg.next();
         }
         cp_async_commit();
@@ -499,7 +513,7 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(CnnWgradArgs a) {
     int64_t issued = 0, waited = 0;   // tiles whose MMAs were committed, and waited for
     bool ok = true;
     int failed = 0;
-    int row = 0, gbuf = 0;
+    int row = 0, slot = 0, gbuf = 0;
     for (int64_t k = 0; k < nt; ++k) {
         if (row + 3 <= c_prev) cp_async_wait_but_last();
         else cp_async_wait_all();
@@ -509,15 +523,18 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(CnnWgradArgs a) {
         tc_fence_after();
         if (failed) break;
         if (tid == 0) {
-            const uint32_t ab = xb + (row % RING) * SLOT_BYTES, bb = gb + gbuf * WG_SMEM_G;
+            const uint64_t ad = umma_desc(xb + slot * SLOT_BYTES, lbo, sbo_a);
+            const uint64_t bd = umma_desc(gb + gbuf * WG_SMEM_G, lbo, sbo_b);
+#pragma unroll
             for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
                 for (int kc = 0; kc < CNN_TILE / 16; ++kc)
-                    umma_bf16(tmem + (uint32_t)(dx * 32), umma_desc(ab + dx * 16 + kc * 2 * WG_K_STRIDE, lbo, sbo_a),
-                              umma_desc(bb + kc * 2 * WG_K_STRIDE, lbo, sbo_b), idesc, (k > 0 || kc > 0) ? 1u : 0u);
+                    umma_bf16(tmem + (uint32_t)(dx * 32), ad + dx + kc * 2 * WG_K_STRIDE / 16,
+                              bd + kc * 2 * WG_K_STRIDE / 16, idesc, (k > 0 || kc > 0) ? 1u : 0u);
             umma_commit(s_bar + (k & 1));
         }
         ++issued;
-        if (warp < cout / 8) {  // bias gradient
+        if (warp < COUT / 8) {  // bias gradient
             const uint4* g = reinterpret_cast<const uint4*>(s_g + gbuf * WG_SMEM_G) + warp * CNN_TILE + lane;
 #pragma unroll
             for (int q = 0; q < CNN_TILE / 32; ++q) {
@@ -537,14 +554,16 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(CnnWgradArgs a) {
         }
         c_prev = rows.count;
         if (ok) {
-            while (rows.tiles > 0 && rows.count < row + RING) rows.fetch<true>(a.x, cin, xb, tid);
+            while (rows.tiles > 0 && rows.count < row + RING) rows.fetch<CIN, true>(a.x, xb, tid);
             if (gleft > 0) {
-                wgrad_fetch_gy(a.gy, tg, cout, gb + (gbuf == 0 ? 2 : gbuf - 1) * WG_SMEM_G, tid);  // tile k + 2
+                wgrad_fetch_gy<COUT>(a.gy, tg, gb + (gbuf == 0 ? 2 : gbuf - 1) * WG_SMEM_G, tid);  // tile k + 2
                 if (--gleft > 0) tg.next();
             }
         }
         cp_async_commit();
-        row += t.next() ? 3 : 1;
+        const int step = t.next() ? 3 : 1;
+        row += step;
+        slot = slot + step >= RING ? slot + step - RING : slot + step;
         gbuf = gbuf == WG_GBUF - 1 ? 0 : gbuf + 1;
     }
     // the last tile's MMAs (after a failed wait, all that may still be in flight)
@@ -557,26 +576,25 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(CnnWgradArgs a) {
     tc_fence_before();
     failed |= __syncthreads_or(!ok);
     tc_fence_after();
-    const int nent = 9 * cin * cout;
-    float* dst = a.part + (int64_t)blockIdx.x * (nent + cout);
+    constexpr int nent = 9 * CIN * COUT;
+    float* dst = a.part + (int64_t)blockIdx.x * (nent + COUT);
     if (nt > 0 && !failed) {
         // warp w holds TMEM lanes 32w..32w+31 = row w of the window (tap row dy = w), channel = lane
         for (int dx = 0; dx < 3; ++dx) {
-            float v[32];
+            float v[COUT];
             const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(dx * 32);
-            if (cout == 32) tmem_ld_x32(taddr, v);
+            if constexpr (COUT == 32) tmem_ld_x32(taddr, v);
             else tmem_ld_x16(taddr, v);
-            if (warp < 3 && lane < cin) {
-                float4* o = reinterpret_cast<float4*>(dst + ((int64_t)(warp * 3 + dx) * cin + lane) * cout);
+            if (warp < 3 && lane < CIN) {
+                float4* o = reinterpret_cast<float4*>(dst + ((warp * 3 + dx) * CIN + lane) * COUT);
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    if (q < cout / 4) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                for (int q = 0; q < COUT / 4; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
             }
         }
     } else {
         for (int e = tid; e < nent; e += blockDim.x) dst[e] = 0.0f;
     }
-    if (warp < cout / 8)
+    if (warp < COUT / 8)
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             float v = bacc[j];
@@ -590,6 +608,22 @@ __global__ void __launch_bounds__(128) k_wgrad_tc(CnnWgradArgs a) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncol));
 }
 
+// The instance for a layer's channel counts (16 or 32 each) and epilogue.
+static auto wgrad_kernel(int cin, int cout) {
+    return cin == 16 ? (cout == 16 ? k_wgrad_tc<16, 16> : k_wgrad_tc<16, 32>)
+                     : (cout == 16 ? k_wgrad_tc<32, 16> : k_wgrad_tc<32, 32>);
+}
+template <int EPI>
+static auto conv_kernel_of(int cin, int cout) {
+    return cin == 16 ? (cout == 16 ? k_conv_tc<16, 16, EPI> : k_conv_tc<16, 32, EPI>)
+                     : (cout == 16 ? k_conv_tc<32, 16, EPI> : k_conv_tc<32, 32, EPI>);
+}
+static auto conv_kernel(int cin, int cout, int epi) {
+    return epi == EPI_RELU_BF16 ? conv_kernel_of<EPI_RELU_BF16>(cin, cout)
+         : epi == EPI_F32_CH0   ? conv_kernel_of<EPI_F32_CH0>(cin, cout)
+                                : conv_kernel_of<EPI_MASK_BF16>(cin, cout);
+}
+
 cudaError_t cnn_wgrad_tc(const CnnWgradArgs& a, int nblocks, cudaStream_t s, const char** why) {
     *why = "";
     if (a.ntiles <= 0 || nblocks <= 0) return cudaSuccess;
@@ -597,16 +631,25 @@ cudaError_t cnn_wgrad_tc(const CnnWgradArgs& a, int nblocks, cudaStream_t s, con
         *why = "unsupported channel counts";
         return cudaErrorInvalidValue;
     }
-    k_wgrad_tc<<<nblocks, 128, SMEM_WGRAD, s>>>(a);
+    wgrad_kernel(a.cin, a.cout)<<<nblocks, 128, SMEM_WGRAD, s>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) *why = "weight-gradient launch";
     return e;
 }
 
 cudaError_t cnn_conv_init() {
-    cudaError_t e = cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_CONV);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_WGRAD);
+    for (int cin : {16, 32})
+        for (int cout : {16, 32}) {
+            for (int epi : {EPI_RELU_BF16, EPI_F32_CH0, EPI_MASK_BF16}) {
+                const cudaError_t e = cudaFuncSetAttribute(conv_kernel(cin, cout, epi),
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_CONV);
+                if (e != cudaSuccess) return e;
+            }
+            const cudaError_t e = cudaFuncSetAttribute(wgrad_kernel(cin, cout),
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_WGRAD);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
 }
 
 cudaError_t cnn_conv_fwd(const CnnConvArgs& a, int nsm, cudaStream_t s, const char** why) {
@@ -622,7 +665,7 @@ cudaError_t cnn_conv_fwd(const CnnConvArgs& a, int nsm, cudaStream_t s, const ch
         return cudaErrorInvalidValue;
     }
     const int grid = (int)std::min<int64_t>(a.ntiles, (int64_t)std::max(nsm, 1) * CONV_CTAS_PER_SM);
-    k_conv_tc<<<grid, 128, SMEM_CONV, s>>>(a);
+    conv_kernel(a.cin, a.cout, a.epi)<<<grid, 128, SMEM_CONV, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) *why = "kernel launch";
     return e;
