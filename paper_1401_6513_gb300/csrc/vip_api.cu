@@ -13,6 +13,7 @@
 #include <cstring>
 #include <new>
 
+#include "vip_direct.cuh"
 #include "vip_internal.cuh"
 
 using namespace vip;
@@ -121,23 +122,6 @@ struct StageBuf {
         if (own) cudaFree(p);
     }
 };
-
-// Can a kernel on the context's device read x and write y, n entries each, in place of the
-// caller's arrays?  Both lie in this device's memory from the first to the last entry, are
-// aligned as doubles, and do not overlap.  Host arrays and other devices' go through a StageBuf.
-bool direct_vectors(const vip_ctx* c, const double* x, const double* y, int64_t n) {
-    if (n <= 0 || (reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) % sizeof(double)) return false;
-    if (x < y + n && y < x + n) return false;
-    for (const double* p : {x, x + n - 1, y, y + n - 1}) {
-        cudaPointerAttributes a;
-        if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        if (a.type != cudaMemoryTypeDevice || a.device != c->device) return false;
-    }
-    return true;
-}
 
 vip_status do_step(vip_ctx* c, cudaStream_t s) {
     VIP_CUDA(cudaEventRecord(c->ev[0], s));
@@ -962,7 +946,7 @@ vip_status vip_apply(vip_ctx* c, int which, const double* x, double* y) {
     if (which == VIP_OP_HELM_V) off = R;
     cudaStream_t st = c->stream;
     const int64_t nvec = c->N + (pois ? c->nbordered : 0);
-    if (direct_vectors(c, x, y, nvec)) {
+    if (direct_vectors(c->device, x, y, nvec)) {
         launch_apply(c, S, off, pois, x, y, st);
         VIP_CUDA(cudaGetLastError());
         VIP_CUDA(cudaStreamSynchronize(st));

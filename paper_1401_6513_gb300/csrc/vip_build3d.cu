@@ -24,6 +24,7 @@
 #include <string>
 #include <vector>
 
+#include "vip_direct.cuh"
 #include "../../include/vip.h"
 
 struct vip_3d;
@@ -1967,11 +1968,17 @@ vip_status vip_3d_apply(vip_3d* b, int which, const double* x, double* y) {
     DeviceScope ds(b->device);
     const int64_t N = b->N;
     std::vector<void*> tmp;
+    const Csr& T = b->tab[which];
+    if (vip::direct_vectors(b->device, x, y, N)) {
+        k3_csr_apply<<<blocks_for(N, 256), 256, 0, b->stream>>>(N, T.ptr, T.col, T.val, x, y);
+        V3_CUDA(cudaGetLastError());
+        V3_CUDA(cudaStreamSynchronize(b->stream));
+        return VIP_OK;
+    }
     double *dx = nullptr, *dy = nullptr;
     cudaError_t e = alloc(tmp, &dx, N);
     if (e == cudaSuccess) e = alloc(tmp, &dy, N);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dx, x, N * sizeof(double), cudaMemcpyDefault, b->stream);
-    const Csr& T = b->tab[which];
     if (e == cudaSuccess) {
         k3_csr_apply<<<blocks_for(N, 256), 256, 0, b->stream>>>(N, T.ptr, T.col, T.val, dx, dy);
         e = cudaGetLastError();

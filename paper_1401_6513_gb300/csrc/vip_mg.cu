@@ -343,40 +343,109 @@ __global__ void __launch_bounds__(512) k_band_factor(const BandMat* __restrict__
 }
 
 // Columns of B's inverse by substitution, one warp per column j of the unit matrix: forward
-// from the first step that can reach j, back through U's columns.  3 m^2 b multiply-adds,
-// bound by the FP64 unit and the latency of a step: 3.3 ms for 2,145 unknowns.  The columns of a block are far
-// apart: those at the front take twice the steps of those at the end.
-__global__ void __launch_bounds__(512) k_band_solve(const BandMat* __restrict__ mats, const double* __restrict__ ab,
-                                                    const int32_t* __restrict__ piv, const int32_t* __restrict__ top,
-                                                    const double* __restrict__ udi, double* x) {
+// from the first step that can reach j, back through U's columns.  The part of the column that
+// the steps still change lies in a ring in shared memory (ring entries, a power of two that
+// holds 2 b + 64 rows); finished rows go to memory, and the next ones come from it, 32 at a
+// time.  A step's column of the factor is read one step ahead.  3 m^2 b multiply-adds, bound by
+// the FP64 unit: 1.8 ms for 2,145 unknowns (3.3 with the column in memory).  The columns of
+// a block are far apart: those at the front take twice the steps of those at the end.
+__global__ void k_band_solve(const BandMat* __restrict__ mats, const double* __restrict__ ab,
+                             const int32_t* __restrict__ piv, const int32_t* __restrict__ top,
+                             const double* __restrict__ udi, double* x, int ring) {
+    extern __shared__ double s_ring[];
     const BandMat B = mats[blockIdx.y];
-    const int m = B.m, b = B.b, lane = threadIdx.x & 31;
+    const int m = B.m, b = B.b, lane = threadIdx.x & 31, mask = ring - 1;
     const int j = blockIdx.x + (threadIdx.x >> 5) * gridDim.x;
     if (j >= m) return;
     const double* M = ab + B.ab + 2 * b;
     const int64_t cs = B.ld - 1;
     double* X = x + B.x + (int64_t)j * m;
-    for (int i = lane; i < m; i += 32) X[i] = i == j ? 1.0 : 0.0;
+    double* w = s_ring + (threadIdx.x >> 5) * ring;
+    constexpr int PRE = 3;                     // prefetched entries a lane (all of them up to b = 96)
+    double pre[PRE];
+    const int k0 = max(0, j - b);
+    for (int i = lane; i < k0; i += 32) X[i] = 0.0;
+    for (int i = k0 + lane; i <= min(k0 + b, m - 1); i += 32) w[i & mask] = i == j ? 1.0 : 0.0;
+    auto column = [&](int k) {                 // multipliers of step k
+#pragma unroll
+        for (int t = 0; t < PRE; ++t) {
+            const int i = lane + 32 * t;
+            pre[t] = k < m && i < min(b, m - 1 - k) ? __ldg(M + k * cs + k + 1 + i) : 0.0;
+        }
+    };
+    column(k0);
+    int p = piv[B.row + k0], done = k0;        // rows below done are in memory
     __syncwarp();
-    for (int k = max(0, j - b); k < m; ++k) {
-        const int p = piv[B.row + k];
-        const double c = X[p], a = X[k];
+    for (int k = k0; k < m; ++k) {
+        const double c = w[p & mask], a = w[k & mask];
+        const int nb = min(b, m - 1 - k), pk = p;
+        double l[PRE];
+#pragma unroll
+        for (int t = 0; t < PRE; ++t) l[t] = pre[t];
+        column(k + 1);
+        if (k + 1 < m) p = piv[B.row + k + 1];
         __syncwarp();
-        if (lane == 0 && p != k) { X[k] = c; X[p] = a; }
+        if (lane == 0) {
+            if (pk != k) { w[k & mask] = c; w[pk & mask] = a; }
+            w[(k + 1 + b) & mask] = 0.0;       // the row that the next step reaches
+        }
         __syncwarp();
-        const int nb = min(b, m - 1 - k);
-        const double* l = M + k * cs + k + 1;
-        for (int i = lane; i < nb; i += 32) X[k + 1 + i] -= l[i] * c;
+#pragma unroll
+        for (int t = 0; t < PRE; ++t) {
+            const int i = lane + 32 * t;
+            if (i < nb) w[(k + 1 + i) & mask] -= l[t] * c;
+        }
+        for (int i = lane + 32 * PRE; i < nb; i += 32) w[(k + 1 + i) & mask] -= __ldg(M + k * cs + k + 1 + i) * c;
         __syncwarp();
+        if (k - done == 31 || k == m - 1) {
+            if (done + lane <= k) X[done + lane] = w[(done + lane) & mask];
+            done = k + 1;
+        }
     }
+    __syncwarp();
+    // rows at and above low are in the ring; rows above done + 31 are final and in memory
+    int low = max(0, m - 2 * b - 32);
+    for (int i = low + lane; i < m; i += 32) w[i & mask] = X[i];
+    done = m - 1;
+    int t0 = top[B.row + m - 1];
+    double r = udi[B.row + m - 1];
+    auto ucolumn = [&](int k, int t) {
+#pragma unroll
+        for (int q = 0; q < PRE; ++q) {
+            const int i = t + lane + 32 * q;
+            pre[q] = i < k ? __ldg(M + k * cs + i) : 0.0;
+        }
+    };
+    ucolumn(m - 1, t0);
+    __syncwarp();
     for (int k = m - 1; k >= 0; --k) {
-        const int t = top[B.row + k];
-        const double c = X[k] * udi[B.row + k];
-        const double* u = M + k * cs;
+        const double c = w[k & mask] * r;
+        const int t = t0;
+        double u[PRE];
+#pragma unroll
+        for (int q = 0; q < PRE; ++q) u[q] = pre[q];
+        if (k > 0) {
+            t0 = top[B.row + k - 1];
+            r = udi[B.row + k - 1];
+            ucolumn(k - 1, t0);
+        }
         __syncwarp();
-        if (lane == 0) X[k] = c;
-        for (int i = t + lane; i < k; i += 32) X[i] -= u[i] * c;
+        if (lane == 0) w[k & mask] = c;
+#pragma unroll
+        for (int q = 0; q < PRE; ++q) {
+            const int i = t + lane + 32 * q;
+            if (i < k) w[i & mask] -= u[q] * c;
+        }
+        for (int i = t + lane + 32 * PRE; i < k; i += 32) w[i & mask] -= __ldg(M + k * cs + i) * c;
         __syncwarp();
+        if (done - k == 31 || k == 0) {
+            if (done - lane >= k) X[done - lane] = w[(done - lane) & mask];
+            done = k - 1;
+            const int i = low - 1 - lane;      // (into the slots of rows just written, or free ones)
+            if (i >= 0) w[i & mask] = X[i];
+            low = max(0, low - 32);
+            __syncwarp();
+        }
     }
 }
 
@@ -443,7 +512,7 @@ static vip_status band_inverses(vip_ctx* c, Multigrid& M, const MgLevel& lc, std
     };
     for (size_t g0 = 0, g1; g0 < mats.size(); g0 = g1) {
         int64_t nab = 0, nx = 0, r0 = mats[g0].row, nr = 0;
-        int mmax = 0;
+        int mmax = 0, bmax = 0;
         for (g1 = g0; g1 < mats.size() && g1 - g0 < 65535; ++g1) {
             BandMat& B = mats[g1];
             const int64_t a = (int64_t)B.m * B.ld, q = (int64_t)B.m * B.m;
@@ -451,6 +520,7 @@ static vip_status band_inverses(vip_ctx* c, Multigrid& M, const MgLevel& lc, std
             B.ab = nab; B.x = nx; B.row -= r0;
             nab += a; nx += q; nr += B.m;
             mmax = std::max(mmax, B.m);
+            bmax = std::max(bmax, B.b);
         }
         const int n = (int)(g1 - g0);
         // one allocation: matrices, bands, columns, reciprocal pivots, three integer arrays
@@ -468,7 +538,13 @@ static vip_status band_inverses(vip_ctx* c, Multigrid& M, const MgLevel& lc, std
         VIP_CUDA(cudaGetLastError());
         k_band_factor<<<n, 512, 0, st>>>(dm, ab, piv, top, udi);
         VIP_CUDA(cudaGetLastError());
-        k_band_solve<<<dim3((mmax + 15) / 16, n), 512, 0, st>>>(dm, ab, piv, top, udi, x);
+        // 16 columns a block, fewer where their rings do not fit (128 KB)
+        int ring = 64;
+        while (ring < 2 * bmax + 64) ring *= 2;
+        const int warps = std::max(1, std::min(16, (1 << 14) / ring));
+        const size_t dyn = (size_t)warps * ring * sizeof(double);
+        VIP_CUDA(cudaFuncSetAttribute(k_band_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+        k_band_solve<<<dim3((mmax + warps - 1) / warps, n), 32 * warps, dyn, st>>>(dm, ab, piv, top, udi, x, ring);
         VIP_CUDA(cudaGetLastError());
         k_band_store<<<dim3((unsigned)std::min<int64_t>(((int64_t)mmax * mmax + 255) / 256, 1024), n), 256, 0, st>>>(
             dm, dpos, x, M.cinv, M.cinv32);
