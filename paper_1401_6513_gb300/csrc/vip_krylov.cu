@@ -51,6 +51,14 @@
 namespace vip {
 
 constexpr int NT64 = 512, NT32 = 512;  // threads of the launch's CTAs (one per SM): FP64 and FP32 iteration
+// The all-FP64 form takes twice the threads where an iteration streams LARGE_STREAM operator
+// entries or more (those of slices without a shared stencil): there the stream and the FP64 unit
+// bound it, and more loads in flight outweigh the spills.  Milliseconds per iteration with 512
+// and 1,024 threads: 2.7M rows of triangular cavities (36M entries) 1.69 and 1.54, 1.9M rows
+// (26M) 1.20 and 1.12, 0.67M rows (9M) 0.523 and 0.527; 2.1M rows of a lattice (0.7M entries)
+// 0.71 and 0.74.
+constexpr int NT64_LARGE = 1024;
+constexpr int64_t LARGE_STREAM = 16000000;
 constexpr int MAXSYS = 128;
 constexpr int KSMEM_TILE = (36 * 36 + 32 * 32) * (int)sizeof(double);  // a coarse tile and its halo, its own cells
 // per-thread dot-product sums: RED_SLOTS systems x RED_Q quantities x NT values of T,
@@ -1496,6 +1504,7 @@ vip_status krylov_plan(vip_ctx* c, KrylovPlan& P, const Sell& A, const std::vect
     {
         struct { const void* k; int nt, dyn; } kern[] = {
             {(const void*)k_bicgstab<double, double, NT64>, NT64, dyn_bytes<double, double, NT64>()},
+            {(const void*)k_bicgstab<double, double, NT64_LARGE>, NT64_LARGE, dyn_bytes<double, double, NT64_LARGE>()},
             {(const void*)k_bicgstab<float, float, NT32>, NT32, dyn_bytes<float, float, NT32>()},
             {(const void*)k_bicgstab<double, float, NT64>, NT64, dyn_bytes<double, float, NT64>()}};
         for (const auto& k : kern) {
@@ -1669,6 +1678,8 @@ vip_status krylov_solve(vip_ctx* c, const KrylovPlan& P, const Sell& A, const do
         return launch<float, float, NT32>(c, P, A, b, x, rtol, max_iters, inner_rtol, mg);
     if (precision == VIP_PREC_MG32 && mg && mg->built)
         return launch<double, float, NT64>(c, P, A, b, x, rtol, max_iters, inner_rtol, mg);
+    if (A.nstored_other >= LARGE_STREAM)
+        return launch<double, double, NT64_LARGE>(c, P, A, b, x, rtol, max_iters, inner_rtol, mg);
     return launch<double, double, NT64>(c, P, A, b, x, rtol, max_iters, inner_rtol, mg);
 }
 
