@@ -35,12 +35,16 @@
 // operation takes about 0.1 us on this part) and instruction fetches: the launch's code
 // is larger than the instruction caches, so what every iteration executes is kept in one
 // copy (one V-cycle and one operator application for both half steps, reductions and
-// barriers as calls: 400 -> 220 KB of instructions).  512 threads with 128 registers
-// beat 384, 640, 768 and 1024 on every size tried (2.1M rows in FP32: 0.39 ms per
-// iteration against 0.44, 0.43, 0.49 and 0.53; the wider ones spill).  Microseconds per
-// iteration, before and now: 4,096 rows FP64 97 -> 70, 65,536 rows FP64 138 -> 112,
-// 525,065 rows FP32 191 -> 140, 2.1M rows FP32 470 -> 345, 16 triangular cavities FP64
-// 250 -> 240.
+// barriers as calls: 220 KB of instructions, 400 in two copies).  512 threads with 128
+// registers beat 384, 640 and 768 (2.1M rows in FP32: 0.39 ms per iteration against 0.44,
+// 0.43 and 0.49) and, but for the sets of LARGE_STREAM, 1,024.  A row's entries come a warp's
+// item ahead into L2 by two bulk prefetches, which hold no registers.  The FP64 unit (two
+// lanes per clock) bounds the coarse tiles and half of a fine pass, so FP64 sums hold no
+// operation but their products.  Microseconds per Poisson iteration (in brackets: 1,024 threads
+// of 64 registers for every set, one row per lane, no work items): 4,096 rows FP64 70 (96), 65,536 rows FP64
+// 110 (136), 525,065 rows FP32 132 (198), 2.1M rows FP32 314 (477); triangular cavities in FP64,
+// all active: 16 of 217,425 rows 226 (246), 20 of 671,018 477 (498), 64 of 2.7M 1398 (1461); the
+// last with an FP32 V-cycle 1076 (1124).
 #include <cstdio>
 #include <cstring>
 #include <type_traits>
@@ -51,14 +55,21 @@
 namespace vip {
 
 constexpr int NT64 = 512, NT32 = 512;  // threads of the launch's CTAs (one per SM): FP64 and FP32 iteration
-// The all-FP64 form takes twice the threads where an iteration streams LARGE_STREAM operator
-// entries or more (those of slices without a shared stencil): there the stream and the FP64 unit
-// bound it, and more loads in flight outweigh the spills.  Milliseconds per iteration with 512
-// and 1,024 threads: 2.7M rows of triangular cavities (36M entries) 1.69 and 1.54, 1.9M rows
-// (26M) 1.20 and 1.12, 0.67M rows (9M) 0.523 and 0.527; 2.1M rows of a lattice (0.7M entries)
-// 0.71 and 0.74.
+// A preconditioned FP64 iteration takes twice the threads where it streams LARGE_STREAM operator
+// entries or more (those of slices without a shared stencil): the entries then come from memory
+// beyond L2 in every pass, and twice the warps hide more of that than the wider batches of fewer
+// warps.  The form has 64 registers a thread, so it keeps the plain row loop only (no four-slice
+// items, no rows shared by lanes), loads a tile's coefficients when it needs them and sums b_1
+// in a phase of its own.  Microseconds per iteration with 512 and 1,024 threads, all FP64: 0.67M
+// rows of triangular cavities (9.2M entries) 477 and 480, 1.9M rows (27M) 1072 and 1004, 2.7M
+// rows (39M) 1507 and 1398; with an FP32 V-cycle 367 and 380, 865 and 762, 1208 and 1076.
+// Without a preconditioner (Helmholtz, a fifth of the passes) 512 threads stay ahead: 253
+// and 260, 383 and 404.
 constexpr int NT64_LARGE = 1024;
-constexpr int64_t LARGE_STREAM = 16000000;
+#ifndef VIP_LARGE_STREAM   // (set by the tests)
+#define VIP_LARGE_STREAM 16000000
+#endif
+constexpr int64_t LARGE_STREAM = VIP_LARGE_STREAM;
 constexpr int MAXSYS = 128;
 constexpr int KSMEM_TILE = (36 * 36 + 32 * 32) * (int)sizeof(double);  // a coarse tile and its halo, its own cells
 // per-thread dot-product sums: RED_SLOTS systems x RED_Q quantities x NT values of T,
@@ -333,7 +344,10 @@ __device__ __forceinline__ void stp(T* p, const Pack<T, N>& q) {
 // to its warps in turn.  (Slices dealt in turn instead put every boundary slice of a
 // lattice whose rows are a multiple of the warps' stride long on the same warp: 38 us per
 // pass on the h = 1/64 bumpy channel, whose row is 64 slices, against 13 with items.)
-constexpr int ITEM_CAP = 768;
+#ifndef VIP_ITEM_CAP   // (set by the tests)
+#define VIP_ITEM_CAP 768
+#endif
+constexpr int ITEM_CAP = VIP_ITEM_CAP;
 __device__ __forceinline__ int64_t entries_at(const int4 si) {  // sell_part's `at` of a slice record
     return si.z >= 0 ? (int64_t)si.z : ~((int64_t)si.y << 32 | (uint32_t)si.x);
 }
@@ -609,13 +623,14 @@ __device__ __noinline__ TileMeta tile_meta(const MgDev<TM>& M, int l, int64_t t)
 template <class T, class TM, int NT>
 __global__ void __launch_bounds__(NT, 1) k_bicgstab(KArgs<T, TM> a) {
     constexpr int KTHREADS = NT, KWARPS = NT / 32;
+    constexpr bool LARGE = NT > NT64;  // the streaming form: 64 registers a thread, so the plain row loop only
     constexpr int TROWS = (32 + KWARPS - 1) / KWARPS;  // rows of a 32-row coarse tile per warp
-    constexpr int ROW_U = sizeof(T) == 8 ? 7 : 14;  // entries of a row in flight
     // |r_hat . r| below this fraction of ||r_hat|| ||r|| is rounding noise in T
     // (FP32 vectors of ~1e6 rows: ~6e-8 / sqrt(n) relative noise in a dot product)
     const double bd_tol = sizeof(T) == 8 ? 1e-14 : 1e-9;
     constexpr bool K32 = std::is_same_v<T, float>;   // FP32 Krylov iteration
     constexpr bool M32 = std::is_same_v<TM, float>;  // FP32 V-cycle
+    constexpr bool fold = M32 && !LARGE;             // level 1 goes down straight from the fine residual
 
     constexpr int V = 16 / (int)sizeof(T);  // rows per thread of the streaming phases
 
@@ -725,7 +740,7 @@ __global__ void __launch_bounds__(NT, 1) k_bicgstab(KArgs<T, TM> a) {
             } else {
 #pragma unroll
                 for (int k = 0; k < RED_Q; ++k)
-                    warp_add(dot_t ? (double)qacck[k] : qacc[k], sacc + (qj * NQ + k) * KWARPS + warp);
+                    warp_add(!K32 || dot_t ? (double)qacck[k] : qacc[k], sacc + (qj * NQ + k) * KWARPS + warp);
             }
         }
         qj = -1;
@@ -809,6 +824,7 @@ __global__ void __launch_bounds__(NT, 1) k_bicgstab(KArgs<T, TM> a) {
     auto fine = [&](const auto* vec, const auto* A, const auto* uA, auto diff, auto&& on, int nq, auto&& pre, auto&& epi) {
         using TA = std::remove_cv_t<std::remove_pointer_t<decltype(vec)>>;
         constexpr bool D = decltype(diff)::value;
+        constexpr int ROW_U = sizeof(TA) == 8 ? (LARGE ? 5 : 7) : (LARGE ? 8 : 14);  // entries of a row in flight
         constexpr int LANES4 = sizeof(TA) == 8 ? KWARPS / 4 : KWARPS / 2, LANES2 = sizeof(TA) == 8 ? KWARPS / 2 : 2 * KWARPS;
         auto ld = [&](int j) -> TA { return ldv(vec + j); };
         auto rs = [&](int64_t row) -> TA {
@@ -816,7 +832,7 @@ __global__ void __launch_bounds__(NT, 1) k_bicgstab(KArgs<T, TM> a) {
             else return (TA)0;
         };
         const bool listed = P.item0[0] >= 0;
-        if (P.nv > LANES2 || P.mixed) {
+        if (LARGE || P.nv > LANES2 || P.mixed) {
             const int i1 = listed ? P.item0[P.nseg] : P.nv;
             int gon = -1;  // system of the item before
             bool is_on = false;
@@ -837,7 +853,17 @@ __global__ void __launch_bounds__(NT, 1) k_bicgstab(KArgs<T, TM> a) {
                     if (nq && is_on) enter(g, nq);
                 }
                 if (!is_on) continue;
-                if (c == 4) {
+                // the warp's next item on its way to L2 (no register waits for it)
+                if (listed && i + KWARPS < i1) {
+                    const int4 nx = s_items[i + KWARPS];
+                    const uint32_t n = (uint32_t)((nx.y >> 3) & SINFO_WIDTH) * SLICE;
+                    if (nx.w < 0 && n && lane < 2) {
+                        const int64_t e = ~((int64_t)nx.w << 32 | (uint32_t)nx.z);
+                        if (lane == 0) l2_prefetch(a.col + e, n * (uint32_t)sizeof(int32_t));
+                        else l2_prefetch(A + e, n * (uint32_t)sizeof(TA));
+                    }
+                }
+                if (!LARGE && c == 4) {
                     const int64_t r0 = (int64_t)it.x * SLICE + lane;
                     TA sum[4], xi[4];
                     decltype(pre((int64_t)0)) pr[4];
@@ -931,8 +957,9 @@ __global__ void __launch_bounds__(NT, 1) k_bicgstab(KArgs<T, TM> a) {
     // memory and little work, so everything that does not depend on the staged iterate
     // (3 x 3 coefficients, right-hand side, step, the fine rows of level 1) is loaded
     // with it, and the tiles' descriptors are kept in shared memory for the launch.
-    // Going down in FP32, level 1 forms b_1 from the fine residual itself (in FP64 the
-    // halo's sums would cost the narrow unit more than the phase saves), and a tile's
+    // Going down in FP32 (fold), level 1 forms b_1 from the fine residual itself; in FP64 the
+    // halo's sums would cost the narrow unit more than the phase saves, and at the 1,024-thread
+    // form's sizes more memory trips (64 cavities: 61 us against 13 + 38).  A tile's
     // residuals are summed over 2 x 2 children straight into b_{l+1}; going up, level 1 adds
     // corr y_1 to the fine rows of each cell directly (y_1 is not stored).  The smoothing
     // steps w D^{-1} are precomputed per omega.  Only rows of systems still in their
@@ -981,9 +1008,9 @@ __global__ void __launch_bounds__(NT, 1) k_bicgstab(KArgs<T, TM> a) {
                 const TM* cp = M.coefs[l] + (c >> 5) * 800 + (c & 31);
                 rg[k] = __ldg(M.ring[l] + (c >> 5));
 #pragma unroll
-                for (int o = 0; o < 9; ++o) co[k][o] = ldm(cp + ((1 + o / 3) * 5 + 1 + o % 3) * 32);
+                for (int o = 0; o < (LARGE ? 0 : 9); ++o) co[k][o] = ldm(cp + ((1 + o / 3) * 5 + 1 + o % 3) * 32);
                 wd[k] = __ldg(wdl + c);
-                if (!M32 || !down || l > 1) bc[k] = ldv(bl + c);
+                if (!down || l > 1 || !fold) bc[k] = ldv(bl + c);
             }
         }
         const int nst = 36 * (th + 4);
@@ -1002,7 +1029,7 @@ __global__ void __launch_bounds__(NT, 1) k_bicgstab(KArgs<T, TM> a) {
                     if (!down) {
                         v[h] = __ldg(wdl + j) * ldv(bl + j) +
                                mcorr * ldv(sol + m.poff + (int64_t)(yy >> 1) * m.psx + (xx >> 1));
-                    } else if (!M32 || l > 1) {
+                    } else if (l > 1 || !fold) {
                         v[h] = __ldg(wdl + j) * ldv(bl + j);
                     } else {
                         const TM b = cell_sum(j);
@@ -1030,14 +1057,20 @@ __global__ void __launch_bounds__(NT, 1) k_bicgstab(KArgs<T, TM> a) {
             if (in[k]) {
                 const int x = m.x0 + lane, y = m.y0 + r;
                 const int64_t c = m.off + (int64_t)y * m.sx + x;
-                TM acc[3];  // one chain per stencil row
+                const TM* cp = M.coefs[l] + (c >> 5) * 800 + (c & 31);
+                if constexpr (LARGE) {
 #pragma unroll
-                for (int dy = 0; dy < 3; ++dy) {
-                    const TM* t = s_tile + (r + 1 + dy) * 36 + lane + 1;
-                    acc[dy] = co[k][3 * dy] * t[0] + co[k][3 * dy + 1] * t[1] + co[k][3 * dy + 2] * t[2];
+                    for (int o = 0; o < 9; ++o) co[k][o] = ldm(cp + ((1 + o / 3) * 5 + 1 + o % 3) * 32);
                 }
-                if (outer) {
-                    const TM* cp = M.coefs[l] + (c >> 5) * 800 + (c & 31);
+                if (fold && down && l == 1) bc[k] = s_tile2[r * 32 + lane];
+                TM res = bc[k];
+                if constexpr (M32) {
+                    TM acc[3];  // one chain per stencil row
+#pragma unroll
+                    for (int dy = 0; dy < 3; ++dy) {
+                        const TM* t = s_tile + (r + 1 + dy) * 36 + lane + 1;
+                        acc[dy] = co[k][3 * dy] * t[0] + co[k][3 * dy + 1] * t[1] + co[k][3 * dy + 2] * t[2];
+                    }
                     TM e[2] = {(TM)0, (TM)0};
 #pragma unroll 1
                     for (uint32_t m2 = outer; m2;) {  // two offsets at a time
@@ -1049,11 +1082,30 @@ __global__ void __launch_bounds__(NT, 1) k_bicgstab(KArgs<T, TM> a) {
                         e[0] += c0 * s_tile[(r + o0 / 5) * 36 + lane + o0 % 5];
                         if (o1 >= 0) e[1] += c1 * s_tile[(r + o1 / 5) * 36 + lane + o1 % 5];
                     }
-                    acc[0] += e[0];
-                    acc[2] += e[1];
+                    if (outer) {
+                        acc[0] += e[0];
+                        acc[2] += e[1];
+                    }
+                    res -= (acc[0] + acc[1]) + acc[2];
+                } else {  // the narrow FP64 unit: no operation but the products
+#pragma unroll
+                    for (int o = 0; o < 9; ++o) res -= co[k][o] * s_tile[(r + 1 + o / 3) * 36 + lane + 1 + o % 3];
+#pragma unroll 1
+                    for (uint32_t m2 = outer; m2;) {  // four offsets at a time
+                        int o[4];
+                        TM q[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            o[u] = m2 ? __ffs(m2) - 1 : -1;
+                            m2 &= m2 - 1;
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) q[u] = o[u] >= 0 ? ldm(cp + o[u] * 32) : (TM)0;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (o[u] >= 0) res -= q[u] * s_tile[(r + o[u] / 5) * 36 + lane + o[u] % 5];
+                    }
                 }
-                if (M32 && down && l == 1) bc[k] = s_tile2[r * 32 + lane];
-                const TM res = bc[k] - ((acc[0] + acc[1]) + acc[2]);
                 if (down) {
                     bc[k] = res;
                 } else {
@@ -1122,7 +1174,7 @@ __global__ void __launch_bounds__(NT, 1) k_bicgstab(KArgs<T, TM> a) {
                  if (own) M.fr[row] = vr - sum;
              });
         if (!grid_sync(a.bar, nb, a.status)) return false;
-        if (!M32 || L == 1) {  // level 1's downward pass does not form b_1
+        if (!fold || L == 1) {  // level 1's downward pass does not form b_1
             for (int64_t c = (int64_t)blockIdx.x * KTHREADS + threadIdx.x; c < M.n[1]; c += (int64_t)nb * KTHREADS)
                 M.b[1][c] = cell_sum(c);
             if (!grid_sync(a.bar, nb, a.status)) return false;
@@ -1506,7 +1558,8 @@ vip_status krylov_plan(vip_ctx* c, KrylovPlan& P, const Sell& A, const std::vect
             {(const void*)k_bicgstab<double, double, NT64>, NT64, dyn_bytes<double, double, NT64>()},
             {(const void*)k_bicgstab<double, double, NT64_LARGE>, NT64_LARGE, dyn_bytes<double, double, NT64_LARGE>()},
             {(const void*)k_bicgstab<float, float, NT32>, NT32, dyn_bytes<float, float, NT32>()},
-            {(const void*)k_bicgstab<double, float, NT64>, NT64, dyn_bytes<double, float, NT64>()}};
+            {(const void*)k_bicgstab<double, float, NT64>, NT64, dyn_bytes<double, float, NT64>()},
+            {(const void*)k_bicgstab<double, float, NT64_LARGE>, NT64_LARGE, dyn_bytes<double, float, NT64_LARGE>()}};
         for (const auto& k : kern) {
             VIP_CUDA(cudaFuncSetAttribute(k.k, cudaFuncAttributeMaxDynamicSharedMemorySize, k.dyn));
             VIP_CUDA(cudaFuncSetAttribute(k.k, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1674,13 +1727,15 @@ static vip_status launch(vip_ctx* c, const KrylovPlan& P, const Sell& A, const d
 vip_status krylov_solve(vip_ctx* c, const KrylovPlan& P, const Sell& A, const double* b, double* x,
                         int precision, double rtol, int32_t max_iters, double inner_rtol,
                         const Multigrid* mg) {
+    const bool use_mg = mg && mg->built;
+    const bool large = use_mg && A.nstored_other >= LARGE_STREAM;
     if (precision == VIP_PREC_MIXED)
         return launch<float, float, NT32>(c, P, A, b, x, rtol, max_iters, inner_rtol, mg);
-    if (precision == VIP_PREC_MG32 && mg && mg->built)
-        return launch<double, float, NT64>(c, P, A, b, x, rtol, max_iters, inner_rtol, mg);
-    if (A.nstored_other >= LARGE_STREAM)
-        return launch<double, double, NT64_LARGE>(c, P, A, b, x, rtol, max_iters, inner_rtol, mg);
-    return launch<double, double, NT64>(c, P, A, b, x, rtol, max_iters, inner_rtol, mg);
+    if (precision == VIP_PREC_MG32 && use_mg)
+        return large ? launch<double, float, NT64_LARGE>(c, P, A, b, x, rtol, max_iters, inner_rtol, mg)
+                     : launch<double, float, NT64>(c, P, A, b, x, rtol, max_iters, inner_rtol, mg);
+    return large ? launch<double, double, NT64_LARGE>(c, P, A, b, x, rtol, max_iters, inner_rtol, mg)
+                 : launch<double, double, NT64>(c, P, A, b, x, rtol, max_iters, inner_rtol, mg);
 }
 
 }  // namespace vip
