@@ -1610,7 +1610,6 @@ vip_status solve_with(vip_3d* b, int kind, double* const* x, int slot) {
         if (!b->work) V3_CUDA(alloc(b->build_bufs, &b->work, pos_bytes<3>() / 8 * 32 * b->nsl));
         a.work = b->work;
     }
-    V3_CUDA(cudaFuncSetAttribute(k3_bicgstab<NS, NT3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
     V3_CUDA(cudaMemsetAsync(b->dbar, 0, sizeof(uint32_t), b->stream));
     void* args[] = {&a};
     V3_CUDA(cudaLaunchCooperativeKernel((const void*)k3_bicgstab<NS, NT3>, dim3(nb), dim3(NT3), args, dyn, b->stream));
@@ -1708,6 +1707,15 @@ vip_status vip_3d_create(vip_3d** out, int device, void* cuda_stream) {
         return VIP_ERR_CUDA;
     }
     b->smem = std::max(0, optin - (int)fa.sharedSizeBytes - 1024);
+    // One limit for every handle on the device: it belongs to the kernel, not to a launch, so a
+    // solve that set it to its own need could lower it under another thread's launch.
+    for (const void* k : {(const void*)k3_bicgstab<1, 256>, (const void*)k3_bicgstab<1, 512>,
+                          (const void*)k3_bicgstab<3, 256>, (const void*)k3_bicgstab<3, 512>})
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, b->smem) != cudaSuccess) {
+            (void)cudaGetLastError();
+            delete b;
+            return VIP_ERR_CUDA;
+        }
     *out = b;
     return VIP_OK;
 }
