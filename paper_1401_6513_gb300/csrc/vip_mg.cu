@@ -538,12 +538,14 @@ static vip_status band_inverses(vip_ctx* c, Multigrid& M, const MgLevel& lc, std
         VIP_CUDA(cudaGetLastError());
         k_band_factor<<<n, 512, 0, st>>>(dm, ab, piv, top, udi);
         VIP_CUDA(cudaGetLastError());
-        // 16 columns a block, fewer where their rings do not fit (128 KB)
+        // 16 columns a block, fewer where their rings do not fit (128 KB; the limit belongs to the
+        // kernel, which other threads' set-ups launch too, so it is the same in every call)
+        constexpr int SOLVE_SMEM = 128 << 10;
         int ring = 64;
         while (ring < 2 * bmax + 64) ring *= 2;
-        const int warps = std::max(1, std::min(16, (1 << 14) / ring));
+        const int warps = std::max(1, std::min(16, SOLVE_SMEM / 8 / ring));
         const size_t dyn = (size_t)warps * ring * sizeof(double);
-        VIP_CUDA(cudaFuncSetAttribute(k_band_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+        VIP_CUDA(cudaFuncSetAttribute(k_band_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, SOLVE_SMEM));
         k_band_solve<<<dim3((mmax + warps - 1) / warps, n), 32 * warps, dyn, st>>>(dm, ab, piv, top, udi, x, ring);
         VIP_CUDA(cudaGetLastError());
         k_band_store<<<dim3((unsigned)std::min<int64_t>(((int64_t)mmax * mmax + 255) / 256, 1024), n), 256, 0, st>>>(
