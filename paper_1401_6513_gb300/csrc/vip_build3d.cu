@@ -15,6 +15,7 @@
 // point's neighbour list is a CSR row (int64 offsets, int32 node indices sorted
 // ascending).  Node points carry 7 weight arrays (the derivative tables), the
 // other points one (interpolation).  Tables are assembled as CSR on first use.
+#include <cuda_pipeline.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -675,89 +676,126 @@ __global__ void k3_scan_add(int64_t* __restrict__ out, int64_t n, const int64_t*
 }
 
 // ---- the fractional step in 3D (Sec. 2, Eqs. 12-15) ----------------------
-// The step reads its tables in slices of 32 rows (SELL-32: entry k of row r at base[r / 32]
-// + 32 k + r % 32), made from the CSR tables and point lists on the first step: a thread
+// The step reads four tables in slices of 32 rows (SELL-32: entry k of the row at position q
+// at base[q / 32] + 32 k + q % 32), made from the point lists on the first step: a thread
 // per row then reads columns and values coalesced, where CSR rows of ~45 entries put the
 // 32 lanes of a warp on 32 lines per entry.  Rows are summed in the same order with the
 // same operations as from CSR, so the sums are the same bits.
+//   0     the solves' system: L at interior rows, the Neumann rows at walls
+//   1..3  Gx, Gy, Gz at interior rows
+// Rows stand in an order of their own (perm): interior rows and wall rows in slices apart,
+// the wall slices spread evenly among the others.  A Neumann row is about twice as long as
+// an interior one, and in node order every lattice line ends in two, so that every slice
+// would be as wide as its wall rows.  The first interior node k0 is at position 0, the
+// border row N at position 1: N's row is k0's own equation, k0's row is empty.
+// All four are laid out with one pass over the rows for the lengths, one scan and one
+// allocation, straight from the point lists (first step with 32^3 and 64^3 nodes 0.7 and 3.4 ms,
+// 8.1 KB of device memory a node; twelve tables copied from CSR took 3.3 and 10.9 ms, 15.6 KB).
+constexpr int NTAB = 4;
 struct Sell3 {
     const int64_t* base = nullptr;    // [slices + 1]
-    const int32_t* len = nullptr;     // [rows] entries of each row
+    const int32_t* len = nullptr;     // [positions] entries of each row
     const int32_t* col = nullptr;
     const double* val = nullptr;
 };
 
-// Source of a step table's rows.
-enum { SRC_CSR = 0, SRC_VIP = 1, SRC_POIS = 2 };
-struct Src3 {
-    int kind, vip;           // SRC_VIP: which of the six VIPs
-    int64_t rows, N, k0;
-    Csr a, nb;               // SRC_CSR: the table; SRC_POIS: L and the Neumann rows
-    const int32_t* perm;     // row of each position (-1: none), or null: position = row
-    Asm A;
-};
-// entries [b, e) of row r, and their arrays
-__device__ __forceinline__ void src_row(const Src3& q, int64_t r, int64_t& b, int64_t& e, const int32_t*& col,
-                                        const double*& val) {
-    b = e = 0;
-    col = q.a.col;
-    val = q.a.val;
-    if (q.perm) r = q.perm[r];
-    if (r < 0 || (q.kind == SRC_CSR && r >= q.N)) return;
-    if (q.kind == SRC_CSR) {
-        b = q.a.ptr[r];
-        e = q.a.ptr[r + 1];
-    } else if (q.kind == SRC_VIP) {
-        const int32_t i = q.A.ipos[r];
-        if (i < 0) return;
-        const int64_t p = q.A.a.N + (int64_t)q.vip * q.A.a.Ni + i;
-        col = q.A.pidx;
-        val = q.A.w0 - q.A.nnz_nodes;
-        b = q.A.pptr[p];
-        e = q.A.pptr[p + 1];
-    } else if (r != q.k0) {  // row k0 holds its diagonal only, row N the equation of k0
-        const bool wall = r < q.N && q.A.ipos[r] < 0;
-        const Csr& t = wall ? q.nb : q.a;
-        const int64_t row = r == q.N ? q.k0 : r;
-        col = t.col;
-        val = t.val;
-        b = t.ptr[row];
-        e = t.ptr[row + 1];
+// perm[q]: row at position q (-1: none).  Slice k holds walls where floor((k + 1) nw / nsl)
+// exceeds floor(k nw / nsl), nw of the nsl slices being walls.
+__global__ void k3_perm(int64_t N, int64_t Ni, int64_t Nb, int64_t nsl, int64_t nw,
+                        const int32_t* __restrict__ interior, const int32_t* __restrict__ boundary,
+                        int32_t* __restrict__ perm) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= 32 * nsl) return;
+    const int64_t k = q >> 5, j = k * nw / nsl;
+    int32_t r = -1;
+    if ((k + 1) * nw / nsl > j) {
+        const int64_t i = 32 * j + (q & 31);
+        if (i < Nb) r = boundary[i];
+    } else {
+        const int64_t i = 32 * (k - j) + (q & 31);   // k0, N, the other interior nodes
+        if (i == 1) r = (int32_t)N;
+        else if (i <= Ni) r = interior[i == 0 ? 0 : i - 1];
     }
+    perm[q] = r;
 }
 
-__global__ void k3_sell_size(Src3 q, int64_t nsl, int32_t* __restrict__ len, int32_t* __restrict__ size) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // whole warps: a slice each
-    if (r >= nsl * 32) return;
+// Entries of row r of table t in column order, f(column, value).
+template <class F>
+__device__ __forceinline__ void step_row(const Asm& A, int t, int64_t r, F f) {
+    if (t > 0) {
+        merge_row(A, VIP3_OP_GX + t - 1, r, f);
+    } else if (A.ipos[r] < 0) {
+        merge_row(A, VIP3_OP_NEUMANN, r, f);
+    } else {
+        for (int64_t s = A.pptr[r]; s < A.pptr[r + 1]; ++s)
+            f(A.pidx[s], __dadd_rn(__dadd_rn(A.wnode[4 * A.nnz_nodes + s], A.wnode[5 * A.nnz_nodes + s]),
+                                   A.wnode[6 * A.nnz_nodes + s]));
+    }
+}
+// row of a position as the tables hold it: N stands for k0's equation, k0 for no row
+__device__ __forceinline__ int64_t row_at(const int32_t* __restrict__ perm, int64_t q, int64_t N, int64_t k0) {
+    const int32_t r = perm[q];
+    return r == N ? k0 : r == k0 ? -1 : r;
+}
+
+// Lengths of the rows of table blockIdx.y, and its slices' sizes in size[t nsl ..]; the system's
+// interior slices once more in size[4 nsl ..] (0 for wall slices).
+__global__ void __launch_bounds__(128) k3_step_size(Asm A, const int32_t* __restrict__ perm, int64_t k0, int64_t nsl,
+                                                    int32_t* __restrict__ len, int32_t* __restrict__ size) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // whole warps: a slice each
+    const int t = blockIdx.y;
+    if (q >= 32 * nsl) return;
+    const int64_t r = row_at(perm, q, A.a.N, k0);
     int n = 0;
-    if (r < q.rows) {
-        int64_t b, e;
-        const int32_t* col;
-        const double* val;
-        src_row(q, r, b, e, col, val);
-        n = (int)(e - b);
-        len[r] = n;
+    bool wall = false;
+    if (r >= 0) {
+        wall = A.ipos[r] < 0;
+        if (t == 0 && !wall) n = (int)(A.pptr[r + 1] - A.pptr[r]);
+        else step_row(A, t, r, [&](int32_t, double) { ++n; });
     }
+    len[t * 32 * nsl + q] = n;
     const int w = __reduce_max_sync(0xffffffffu, n);
-    if ((r & 31) == 0) size[r >> 5] = w * 32;
+    wall = __any_sync(0xffffffffu, wall);
+    if ((q & 31) == 0) {
+        size[t * nsl + (q >> 5)] = w * 32;
+        if (t == 0) size[NTAB * nsl + (q >> 5)] = wall ? 0 : w * 32;
+    }
 }
 
-__global__ void k3_sell_fill(Src3 q, const int64_t* __restrict__ base, int32_t* __restrict__ scol,
-                             double* __restrict__ sval) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t sl = r >> 5;
-    if (sl * 32 >= q.rows) return;
-    int64_t b = 0, e = 0;
-    const int32_t* col = nullptr;
-    const double* val = nullptr;
-    if (r < q.rows) src_row(q, r, b, e, col, val);
-    const int w = (int)((base[sl + 1] - base[sl]) >> 5);
-    for (int k = 0; k < w; ++k) {
-        const int64_t o = base[sl] + 32 * k + (r & 31);
-        const bool in = b + k < e;
-        scol[o] = in ? col[b + k] : 0;
-        sval[o] = in ? val[b + k] : 0.0;
+__global__ void __launch_bounds__(128) k3_step_fill(Asm A, const int32_t* __restrict__ perm, int64_t k0, int64_t nsl,
+                                                    const int64_t* __restrict__ base, int32_t* __restrict__ scol,
+                                                    double* __restrict__ sval) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = blockIdx.y;
+    if (q >= 32 * nsl) return;
+    const int64_t* bt = base + t * nsl + (q >> 5);
+    int64_t o = bt[0] + (q & 31);
+    const int64_t r = row_at(perm, q, A.a.N, k0);
+    if (r >= 0)
+        step_row(A, t, r, [&](int32_t c, double v) {
+            scol[o] = c;
+            sval[o] = v;
+            o += 32;
+        });
+    for (; o < bt[1]; o += 32) {
+        scol[o] = 0;
+        sval[o] = 0.0;
     }
+}
+
+// most[0]: entries of the tables; most[1], most[2]: the most that a solve block's slices hold of
+// the system, of its interior slices.
+__global__ void __launch_bounds__(256) k3_step_most(int64_t nsl, int nb, const int64_t* __restrict__ base,
+                                                    unsigned long long* __restrict__ most) {
+    const int t = threadIdx.x;
+    unsigned long long m[2] = {0, 0};
+    for (int64_t k = t; k < nb; k += blockDim.x)
+        for (int i = 0; i < 2; ++i) {
+            const int64_t* bs = base + (i ? NTAB * nsl : 0);
+            m[i] = max(m[i], (unsigned long long)(bs[nsl * (k + 1) / nb] - bs[nsl * k / nb]));
+        }
+    for (int i = 0; i < 2; ++i) atomicMax(most + 1 + i, m[i]);
+    if (t == 0) most[0] = (unsigned long long)base[NTAB * nsl];
 }
 
 // sum_k a_rk x[f][col_rk] for NF fields through one row, in entry order, one chain per
@@ -817,46 +855,113 @@ struct Fields3 { double* f[3]; };
 // Convection at every node (Sec. 4.1 item 1 in three coordinates): the products
 // of the six VIP interpolations of (u, v, w), differenced across each VIP pair
 // and divided by the pair distance.
-struct Vips3 { Sell3 t[6]; };
-__global__ void __launch_bounds__(128) k3_conv(Asm A, Vips3 T, Fields3 u, Fields3 out) {
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= A.a.N) return;
-    const int32_t i = A.ipos[r];
-    if (i < 0) { out.f[0][r] = out.f[1][r] = out.f[2][r] = 0.0; return; }
-    const double* const x[3] = {u.f[0], u.f[1], u.f[2]};
-    double f[3] = {0.0, 0.0, 0.0};
+//
+// A block takes 32 consecutive interior nodes, a warp for each axis.  The warp copies the 32
+// lists of a VIP to shared memory, CONV_E entries of each at a time and the next ones beside
+// the sums, 16 lanes along a list; there every lane walks its own list.  So the lists need no
+// sliced copy (3.4 KB a node).
+constexpr int CONV_E = 16, CONV_P = 33;   // entries of a list in a chunk; pitch of an entry's 32 lists
+__global__ void __launch_bounds__(96) k3_conv(Asm A, Fields3 u, Fields3 out) {
+    __shared__ double s_val[3][2][CONV_E * CONV_P];
+    __shared__ int32_t s_col[3][2][CONV_E * CONV_P];
+    __shared__ double s_x[3][3][32], s_inv[3][32];
+    const int lane = threadIdx.x & 31, ax = threadIdx.x >> 5;
+    const int64_t i0 = 32 * (int64_t)blockIdx.x, i = i0 + lane, Ni = A.a.Ni;
+    const bool in = i < Ni;
+    double v[2][3], q[2][3], rho;
+    int64_t owner;
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        const int64_t p = A.a.N + (int64_t)(2 * ax + side) * Ni + i, b0 = A.pptr[p - lane];
+        const int b = in ? (int)(A.pptr[p] - b0) : 0, len = in ? (int)(A.pptr[p + 1] - b0) - b : 0;
+        const int32_t* col = A.pidx + b0;
+        const double* val = A.w0 - A.nnz_nodes + b0;
+        const int longest = __reduce_max_sync(0xffffffffu, len);
+        auto copy = [&](int k0) {   // entries k0 .. k0 + 15 of every list
+            const int e = lane & (CONV_E - 1), k = k0 + e, buf = (k0 / CONV_E) & 1;
+#pragma unroll
+            for (int j = 0; j < 32; j += 2) {
+                const int l = j + (lane >> 4), at = __shfl_sync(0xffffffffu, b, l) + k;
+                if (k < __shfl_sync(0xffffffffu, len, l)) {
+                    __pipeline_memcpy_async(&s_col[ax][buf][e * CONV_P + l], col + at, 4);
+                    __pipeline_memcpy_async(&s_val[ax][buf][e * CONV_P + l], val + at, 8);
+                }
+            }
+            __pipeline_commit();
+        };
+        double sum[3] = {0.0, 0.0, 0.0};
+        __syncwarp();
+        copy(0);
 #pragma unroll 1
-    for (int ax = 0; ax < 3; ++ax) {
-        double a[3], b[3], qa[3], qb[3], rho;
-        int64_t owner;
-        sell_sums<3>(T.t[2 * ax], r, x, a);
-        sell_sums<3>(T.t[2 * ax + 1], r, x, b);
-        point_of(A.a, A.a.N + (int64_t)(2 * ax) * A.a.Ni + i, qa, rho, owner);
-        point_of(A.a, A.a.N + (int64_t)(2 * ax + 1) * A.a.Ni + i, qb, rho, owner);
-        const double d = ax == 0 ? qa[0] - qb[0] : ax == 1 ? qa[1] - qb[1] : qa[2] - qb[2];
-        const double inv = 1.0 / fabs(d);
-        const double wa = ax == 0 ? a[0] : ax == 1 ? a[1] : a[2], wb = ax == 0 ? b[0] : ax == 1 ? b[1] : b[2];
+        for (int k0 = 0; k0 < longest; k0 += CONV_E) {
+            __syncwarp();           // the chunk before last has been read
+            copy(k0 + CONV_E);
+            __pipeline_wait_prior(1);
+            __syncwarp();
+            const int buf = (k0 / CONV_E) & 1;
+            const int32_t* sc = s_col[ax][buf] + lane;
+            const double* sv = s_val[ax][buf] + lane;
+            constexpr int U = 8;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) f[c] += (wa * a[c] - wb * b[c]) * inv;
+            for (int h = 0; h < CONV_E; h += U) {
+                double g[3][U];
+#pragma unroll
+                for (int w = 0; w < U; ++w) {
+                    const bool on = k0 + h + w < len;
+                    const int c = on ? sc[(h + w) * CONV_P] : 0;
+#pragma unroll
+                    for (int f = 0; f < 3; ++f) g[f][w] = on ? u.f[f][c] : 0.0;
+                }
+#pragma unroll
+                for (int w = 0; w < U; ++w)
+                    if (k0 + h + w < len) {
+                        const double a = sv[(h + w) * CONV_P];
+#pragma unroll
+                        for (int f = 0; f < 3; ++f) sum[f] = fma(a, g[f][w], sum[f]);
+                    }
+            }
+        }
+        __pipeline_wait_prior(0);
+#pragma unroll
+        for (int f = 0; f < 3; ++f) v[side][f] = sum[f];
+        if (in) point_of(A.a, p, q[side], rho, owner);
     }
+    if (in) {
+        const double d = ax == 0 ? q[0][0] - q[1][0] : ax == 1 ? q[0][1] - q[1][1] : q[0][2] - q[1][2];
+        const double wa = ax == 0 ? v[0][0] : ax == 1 ? v[0][1] : v[0][2],
+                     wb = ax == 0 ? v[1][0] : ax == 1 ? v[1][1] : v[1][2];
+        s_inv[ax][lane] = 1.0 / fabs(d);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) out.f[c][r] = f[c];
+        for (int c = 0; c < 3; ++c) s_x[ax][c][lane] = wa * v[0][c] - wb * v[1][c];
+    }
+    __syncthreads();
+    if (!in) return;
+    double f = 0.0;                                   // warp c: component c, axes in order
+    for (int k = 0; k < 3; ++k) f += s_x[k][ax][lane] * s_inv[k][lane];
+    out.f[ax][A.a.interior[i]] = f;
 }
 
 // Right-hand sides of Eq. (12) times dt of the three components at interior rows:
 // (I + alpha L) u^n - dt (1.5 N^n - 0.5 N^{n-1} + G p^n); wall rows: the node's
 // boundary value.  star gets the solves' initial guess u^n.
-struct Grad3 { Sell3 g[3]; };
-__global__ void __launch_bounds__(128) k3_rhs(int64_t N, Sell3 L, Grad3 G, double alpha, double dt,
-                                              const int32_t* __restrict__ ipos, Fields3 bc, Fields3 u, Fields3 Ncur,
+// Thread per position of the tables; the position of row N takes node k0 (see row_at).
+struct Tabs3 {
+    Sell3 sys, g[3];
+    const int32_t* perm;
+    int64_t n, N, k0;        // positions, nodes, first interior node
+    const int32_t* ipos;
+};
+__global__ void __launch_bounds__(128) k3_rhs(Tabs3 T, double alpha, double dt, Fields3 bc, Fields3 u, Fields3 Ncur,
                                               Fields3 Nprev, const double* __restrict__ p, Fields3 rhs, Fields3 star) {
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= N) return;
-    const bool inside = ipos[r] >= 0;
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= T.n) return;
+    const int64_t r = row_at(T.perm, q, T.N, T.k0);
+    if (r < 0) return;
+    const bool inside = T.ipos[r] >= 0;
     double Lu[3] = {0.0, 0.0, 0.0};
     if (inside) {
         const double* const x[3] = {u.f[0], u.f[1], u.f[2]};
-        sell_sums<3>(L, r, x, Lu);
+        sell_sums<3>(T.sys, q, x, Lu);
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -868,7 +973,7 @@ __global__ void __launch_bounds__(128) k3_rhs(int64_t N, Sell3 L, Grad3 G, doubl
         }
         double Gp[1];
         const double* const x[1] = {p};
-        sell_sums<1>(G.g[c], r, x, Gp);
+        sell_sums<1>(T.g[c], q, x, Gp);
         const double nab = 1.5 * Ncur.f[c][r] - 0.5 * Nprev.f[c][r];
         rhs.f[c][r] = (uc + alpha * Lu[c]) - dt * (nab + Gp[0]);
     }
@@ -877,58 +982,64 @@ __global__ void __launch_bounds__(128) k3_rhs(int64_t N, Sell3 L, Grad3 G, doubl
 // Eq. (13) right-hand side, bordered: b_i = (Gx u* + Gy v* + Gz w*)_i / dt at
 // interior rows, 0 at wall rows, then b_N = b_k0 and b_k0 = 0 (k0 the first
 // interior node).
-__global__ void __launch_bounds__(128) k3_div(int64_t N, Grad3 G, double dt, int64_t k0,
-                                              const int32_t* __restrict__ ipos, Fields3 us, double* __restrict__ b) {
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= N) return;
-    if (ipos[r] < 0) { b[r] = 0.0; return; }          // wall rows: zero normal derivative = 0
+__global__ void __launch_bounds__(128) k3_div(Tabs3 T, double dt, Fields3 us, double* __restrict__ b) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= T.n) return;
+    const int64_t r = row_at(T.perm, q, T.N, T.k0);
+    if (r < 0) return;
+    if (T.ipos[r] < 0) { b[r] = 0.0; return; }        // wall rows: zero normal derivative = 0
     double d[3][1];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const double* const x[1] = {us.f[c]};
-        sell_sums<1>(G.g[c], r, x, d[c]);
+        sell_sums<1>(T.g[c], q, x, d[c]);
     }
-    const double q = (d[0][0] + d[1][0] + d[2][0]) / dt;
-    if (r == k0) { b[N] = q; b[r] = 0.0; }
-    else b[r] = q;
+    const double v = (d[0][0] + d[1][0] + d[2][0]) / dt;
+    if (r == T.k0) { b[T.N] = v; b[r] = 0.0; }
+    else b[r] = v;
 }
 
 // Eqs. (14)-(15): u = u* - dt G phi at interior rows; p = p + phi - alpha L phi
-// at every node.
-__global__ void __launch_bounds__(128) k3_project(int64_t N, Sell3 L, Grad3 G, double alpha, double dt,
-                                                  const int32_t* __restrict__ ipos, const double* __restrict__ phi,
+// at every node (a wall row's L from the point lists: the system has its Neumann row).
+__global__ void __launch_bounds__(128) k3_project(Tabs3 T, Asm A, double alpha, double dt, const double* __restrict__ phi,
                                                   Fields3 us, Fields3 u, double* __restrict__ p) {
-    int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= N) return;
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= T.n) return;
+    const int64_t r = row_at(T.perm, q, T.N, T.k0);
+    if (r < 0) return;
     const double* const x[1] = {phi};
-    const bool inside = ipos[r] >= 0;                 // walls keep their values
+    const bool inside = T.ipos[r] >= 0;               // walls keep their values
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         double g[1] = {0.0};
-        if (inside) sell_sums<1>(G.g[c], r, x, g);
+        if (inside) sell_sums<1>(T.g[c], q, x, g);
         u.f[c][r] = inside ? us.f[c][r] - dt * g[0] : us.f[c][r];
     }
-    double l[1];
-    sell_sums<1>(L, r, x, l);
+    double l[1] = {0.0};
+    if (inside) {
+        sell_sums<1>(T.sys, q, x, l);
+    } else {
+        for (int64_t s = A.pptr[r]; s < A.pptr[r + 1]; ++s)
+            l[0] = fma(__dadd_rn(__dadd_rn(A.wnode[4 * A.nnz_nodes + s], A.wnode[5 * A.nnz_nodes + s]),
+                                 A.wnode[6 * A.nnz_nodes + s]),
+                       phi[A.pidx[s]], l[0]);
+    }
     p[r] = (p[r] + phi[r]) - alpha * l[0];
 }
 
 // ---- the step's linear solves ---------------------------------------------
 // The two systems, applied matrix-free from their tables:
-//   HELM: y = x - alpha L x at interior rows, y = x at wall rows      (n = N, table L)
+//   HELM: y = x - alpha L x at interior rows, y = x at wall rows      (n = N)
 //   POIS: the bordered Poisson system (n = N + 1, x_N = mu): interior rows
 //         y_i = (L x)_i + mu, wall rows y_i = (-6/h_i^2) (Nb x)_i, y_k0 =
-//         (-6/h_k0^2) x_k0, y_N = (L x)_k0 + mu              (table SRC_POIS).
+//         (-6/h_k0^2) x_k0, y_N = (L x)_k0 + mu.
+// Both read table 0; the Helmholtz system passes its wall rows over and takes k0's row from
+// the position of row N, the next one.
 // k3_bicgstab<NS> solves NS right-hand sides of one system in one cooperative launch:
 // unpreconditioned FP64 BiCGSTAB (van der Vorst 1992) to ||b - A x|| <= rtol ||b|| with the
 // oracle's rules: restart with r_hat = r when |r_hat . r| or |r_hat . v| falls below 1e-12
 // of the product of norms, and confirm convergence on the true residual.  x holds the
 // initial guess.
-//
-// The solves' tables hold their rows in an order of their own (perm): interior rows and wall
-// rows in slices apart, the wall slices spread evenly among the others.  A Neumann row is
-// about twice as long as an interior one, and in node order every lattice line ends in two,
-// so that every slice would be as wide as its wall rows.
 //
 // A block owns a run of slices.  The vectors (and the table, if it fits) stay in its shared
 // memory for the whole solve; p and s, which other blocks gather from, also go to global
@@ -957,6 +1068,7 @@ struct Solve3 {
     double alpha, rtol;
     int32_t max_it;
     Sell3 t;
+    const int64_t* copied;   // [nsl + 1] a slice's place among those that a block copies to shared memory
     const int32_t* ipos;
     const double* h;
     const double* rhs[NS];
@@ -1033,12 +1145,16 @@ __global__ void __launch_bounds__(NT3, 1) k3_bicgstab(Solve3<NS> a) {
     const double* val = a.t.val + e0;
     const int32_t* col = a.t.col + e0;
     if (a.mat_smem) {
-        const int ne = (int)(a.t.base[s1] - e0);
+        const int ne = (int)(a.copied[s1] - a.copied[s0]);
         double* sv = sm + (a.vec_smem ? (int64_t)(pos_bytes<NS>() / 8) * pitch : 0);
         int32_t* sc = reinterpret_cast<int32_t*>(sv + ne);
-        for (int k = tid; k < ne; k += NT3) {
-            sv[k] = val[k];
-            sc[k] = col[k];
+        for (int64_t s = s0 + warp; s < s1; s += NW3) {
+            const int o = (int)(a.copied[s] - a.copied[s0]), n = (int)(a.copied[s + 1] - a.copied[s]);
+            const int64_t e = a.t.base[s] - e0;
+            for (int k = lane; k < n; k += 32) {
+                sv[o + k] = val[e + k];
+                sc[o + k] = col[e + k];
+            }
         }
         val = sv;
         col = sc;
@@ -1052,13 +1168,15 @@ __global__ void __launch_bounds__(NT3, 1) k3_bicgstab(Solve3<NS> a) {
         if (a.kind == OPK_POIS && r == a.k0) kind = ROW_PIN;
         if (a.kind == OPK_POIS && kind != ROW_IN) sc = -6.0 / (a.h[r] * a.h[r]);
         const bool none = r < 0 || (a.kind == OPK_HELM ? kind == ROW_WALL : kind == ROW_PIN);
-        pos[i] = Pos3{r, kind, none ? 0 : a.t.len[pos0 + i], (int)(a.t.base[s0 + (i >> 5)] - e0) + (i & 31)};
+        const int next = a.kind == OPK_HELM && r == a.k0 ? 1 : 0;
+        const int64_t at = a.mat_smem ? a.copied[s0 + (i >> 5)] - a.copied[s0] : a.t.base[s0 + (i >> 5)] - e0;
+        pos[i] = Pos3{r, kind, none ? 0 : a.t.len[pos0 + i + next], (int)at + (i & 31) + next};
         scale[i] = sc;
         if (r >= 0)
 #pragma unroll
             for (int q = 0; q < NS; ++q) V(VX, q)[i] = a.x[q][r];
     }
-    auto row_at = [&](int i) -> int { return pos[i].row; };
+    auto row_of = [&](int i) -> int { return pos[i].row; };
     if (tid < NS) S[tid] = Sys3{};  // state S3_RESID
     __syncthreads();
     // A applied to NS gathered vectors at position i
@@ -1127,7 +1245,7 @@ __global__ void __launch_bounds__(NT3, 1) k3_bicgstab(Solve3<NS> a) {
         if (__syncthreads_or(tid < NS && S[tid].state == S3_RESID)) {
             if (!first) {  // the iterate to global memory, where its neighbours gather it
                 for (int i = tid; i < pitch; i += NT3) {
-                    const int r = row_at(i);
+                    const int r = row_of(i);
                     if (r < 0) continue;
 #pragma unroll
                     for (int q = 0; q < NS; ++q)
@@ -1205,7 +1323,7 @@ __global__ void __launch_bounds__(NT3, 1) k3_bicgstab(Solve3<NS> a) {
         for (int half = 0; half < 2; ++half) {
             double d[Q * NS] = {};
             for (int i = tid; i < pitch; i += NT3) {
-                const int r = row_at(i);
+                const int r = row_of(i);
                 if (r < 0) continue;
 #pragma unroll
                 for (int q = 0; q < NS; ++q)
@@ -1264,7 +1382,7 @@ __global__ void __launch_bounds__(NT3, 1) k3_bicgstab(Solve3<NS> a) {
         // x += alpha p + omega s;  r = s - omega t
         double d[Q * NS] = {};
         for (int i = tid; i < pitch; i += NT3) {
-            if (row_at(i) < 0) continue;
+            if (row_of(i) < 0) continue;
 #pragma unroll
             for (int q = 0; q < NS; ++q)
                 if (S[q].state == S3_RUN) {
@@ -1295,7 +1413,7 @@ __global__ void __launch_bounds__(NT3, 1) k3_bicgstab(Solve3<NS> a) {
     for (int i = tid; i < pitch; i += NT3)
 #pragma unroll
         for (int q = 0; q < NS; ++q)
-            if (S[q].zero && row_at(i) >= 0) a.x[q][row_at(i)] = 0.0;
+            if (S[q].zero && row_of(i) >= 0) a.x[q][row_of(i)] = 0.0;
     if (blockIdx.x == 0 && tid < NS) {
         a.out[tid] = Out3{S[tid].it, S[tid].status, S[tid].relres};
         if (S[tid].status) atomicCAS(a.status, 0, S[tid].status);
@@ -1354,10 +1472,11 @@ struct vip_3d {
     uint32_t* dbar = nullptr;                     // [2] barrier word, status
     // the step's tables in slices, made on the first step after a build
     bool sliced = false;
-    Sell3 sl_lap, sl_helm, sl_pois, sl_grad[3], sl_vip[6];
-    int32_t* perm = nullptr;                      // the solves' row order (see Solve3)
+    Sell3 tab3[NTAB];
+    int32_t* perm = nullptr;                      // their row order
+    const int64_t* inner = nullptr;               // [nsl + 1] entries of the system's interior slices before each
     int64_t nsl = 0;                              // its slices
-    int64_t ent_helm = 0, ent_pois = 0;           // most entries of a block's slices
+    int64_t ent_helm = 0, ent_pois = 0;           // most entries of a solve block's slices
     int64_t steps = 0;
     int32_t last_helm = 0, last_poisson = 0;
     double last_poisson_res = 0.0;
@@ -1412,16 +1531,21 @@ struct DeviceScope {
     ~DeviceScope() { if (prev >= 0) cudaSetDevice(prev); }
 };
 
-// out[0..n] = exclusive scan of in[0..n) (out[n] = total); *total_host gets the total.
-vip_status scan_counts(vip_3d* b, const int32_t* in, int64_t n, int64_t* out, int64_t* total_host) {
-    const int64_t nb = std::max<int64_t>(1, (n + SCAN_CHUNK - 1) / SCAN_CHUNK);
-    std::vector<void*> tmp;
-    int64_t* bsum = nullptr;
-    cudaError_t e = alloc(tmp, &bsum, nb);
-    if (e != cudaSuccess) { free_all(tmp); V3_CUDA(e); }
+// out[0..n] = exclusive scan of in[0..n) (out[n] = total); bsum: scan_blocks(n) entries of scratch.
+int64_t scan_blocks(int64_t n) { return std::max<int64_t>(1, (n + SCAN_CHUNK - 1) / SCAN_CHUNK); }
+void enqueue_scan(vip_3d* b, const int32_t* in, int64_t n, int64_t* out, int64_t* bsum) {
+    const int64_t nb = scan_blocks(n);
     k3_scan_local<<<(unsigned)nb, SCAN_T, 0, b->stream>>>(in, n, out, bsum);
     k3_scan_blocks<<<1, SCAN_T, 0, b->stream>>>(bsum, nb, out + n);
     k3_scan_add<<<blocks_for(n, 256), 256, 0, b->stream>>>(out, n, bsum);
+}
+// The same with scratch of its own; *total_host gets the total.
+vip_status scan_counts(vip_3d* b, const int32_t* in, int64_t n, int64_t* out, int64_t* total_host) {
+    std::vector<void*> tmp;
+    int64_t* bsum = nullptr;
+    cudaError_t e = alloc(tmp, &bsum, scan_blocks(n));
+    if (e != cudaSuccess) { free_all(tmp); V3_CUDA(e); }
+    enqueue_scan(b, in, n, out, bsum);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(total_host, out + n, sizeof(int64_t), cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
@@ -1491,84 +1615,45 @@ vip_status assemble(vip_3d* b, int op) {
 // blocks of a solve over n rows: one per SM, at least a slice each
 int solve_blocks(const vip_3d* b) { return (int)std::max<int64_t>(1, std::min<int64_t>(b->sms, b->nsl)); }
 
-// A step table in slices; *most gets the largest entry count of a solve block's slices.
-vip_status slice_table(vip_3d* b, const Src3& q, Sell3& t, int64_t* most) {
-    const int64_t nsl = (q.rows + 31) / 32;
-    int32_t *len = nullptr, *size = nullptr, *col = nullptr;
-    int64_t *base = nullptr, nent = 0;
-    double* val = nullptr;
-    V3_CUDA(alloc(b->build_bufs, &len, q.rows));
-    V3_CUDA(alloc(b->build_bufs, &base, nsl + 1));
-    std::vector<void*> tmp;
-    cudaError_t e = alloc(tmp, &size, nsl);
-    if (e != cudaSuccess) { free_all(tmp); V3_CUDA(e); }
-    k3_sell_size<<<blocks_for(nsl * 32, 256), 256, 0, b->stream>>>(q, nsl, len, size);
-    vip_status st = scan_counts(b, size, nsl, base, &nent);
-    free_all(tmp);
-    if (st != VIP_OK) return st;
-    V3_CUDA(alloc(b->build_bufs, &col, nent));
-    V3_CUDA(alloc(b->build_bufs, &val, nent));
-    k3_sell_fill<<<blocks_for(nsl * 32, 256), 256, 0, b->stream>>>(q, base, col, val);
-    V3_CUDA(cudaGetLastError());
-    t.base = base; t.len = len; t.col = col; t.val = val;
-    if (most) {
-        std::vector<int64_t> hb(nsl + 1);
-        V3_CUDA(cudaMemcpyAsync(hb.data(), base, (nsl + 1) * 8, cudaMemcpyDeviceToHost, b->stream));
-        V3_CUDA(cudaStreamSynchronize(b->stream));
-        const int nb = solve_blocks(b);
-        *most = 0;
-        for (int k = 0; k < nb; ++k) *most = std::max(*most, hb[nsl * (k + 1) / nb] - hb[nsl * k / nb]);
-    }
-    return VIP_OK;
-}
-
+// The step's tables (see Sell3).
 vip_status slice_tables(vip_3d* b) {
     if (b->sliced) return VIP_OK;
-    const int need[5] = {VIP3_OP_LAPLACE, VIP3_OP_GX, VIP3_OP_GY, VIP3_OP_GZ, VIP3_OP_NEUMANN};
-    for (int op : need) V3_TRY(assemble(b, op));
-    Src3 q{};
-    q.A = asm_view(b);
-    q.N = b->N;
-    q.k0 = b->k0;
-    q.kind = SRC_CSR;
-    q.rows = b->N;
-    q.a = b->tab[VIP3_OP_LAPLACE];
-    V3_TRY(slice_table(b, q, b->sl_lap, nullptr));
-    for (int c = 0; c < 3; ++c) {
-        q.a = b->tab[VIP3_OP_GX + c];
-        V3_TRY(slice_table(b, q, b->sl_grad[c], nullptr));
-    }
-    q.kind = SRC_VIP;
-    for (int k = 0; k < 6; ++k) {
-        q.vip = k;
-        V3_TRY(slice_table(b, q, b->sl_vip[k], nullptr));
-    }
-    // the solves' row order: interior rows (and the border row N), wall rows, each padded to
-    // whole slices; wall slice j of nw goes after (j + 1) / nw of the others
-    std::vector<int32_t> ip(b->N), in, wall, perm;
-    V3_CUDA(cudaMemcpyAsync(ip.data(), b->ipos, b->N * 4, cudaMemcpyDeviceToHost, b->stream));
-    V3_CUDA(cudaStreamSynchronize(b->stream));
-    for (int64_t r = 0; r < b->N; ++r) (ip[r] >= 0 ? in : wall).push_back((int32_t)r);
-    in.push_back((int32_t)b->N);
-    for (auto* v : {&in, &wall}) v->resize((v->size() + 31) / 32 * 32, -1);
-    const int64_t ni = (int64_t)in.size() / 32, nw = (int64_t)wall.size() / 32;
-    b->nsl = ni + nw;
-    for (int64_t k = 0, i = 0, j = 0; k < b->nsl; ++k) {
-        const bool w = (k + 1) * nw / b->nsl > j;
-        const int32_t* src = w ? wall.data() + 32 * j++ : in.data() + 32 * i++;
-        perm.insert(perm.end(), src, src + 32);
-    }
-    V3_CUDA(alloc(b->build_bufs, &b->perm, perm.size()));
-    V3_CUDA(cudaMemcpyAsync(b->perm, perm.data(), perm.size() * 4, cudaMemcpyHostToDevice, b->stream));
-    V3_CUDA(cudaStreamSynchronize(b->stream));
-    q.perm = b->perm;
-    q.rows = 32 * b->nsl;
-    q.kind = SRC_CSR;
-    q.a = b->tab[VIP3_OP_LAPLACE];
-    V3_TRY(slice_table(b, q, b->sl_helm, &b->ent_helm));
-    q.kind = SRC_POIS;
-    q.nb = b->tab[VIP3_OP_NEUMANN];
-    V3_TRY(slice_table(b, q, b->sl_pois, &b->ent_pois));
+    const Asm A = asm_view(b);
+    cudaStream_t st = b->stream;
+    const int64_t ni = (b->Ni + 1 + 31) / 32, nw = (b->Nb + 31) / 32, nsl = b->nsl = ni + nw, q = 32 * nsl;
+    int32_t *rows = nullptr, *size = nullptr;
+    int64_t* base = nullptr;
+    V3_CUDA(alloc(b->build_bufs, &rows, (1 + NTAB) * q));                  // perm, lengths
+    V3_CUDA(alloc(b->build_bufs, &base, (NTAB + 1) * nsl + 1 + 3));        // offsets, then k3_step_most's results
+    int32_t *perm = rows, *len = rows + q;
+    int64_t* most = base + (NTAB + 1) * nsl + 1;
+    const int64_t nb = scan_blocks((NTAB + 1) * nsl);
+    std::vector<void*> tmp;
+    cudaError_t e = alloc(tmp, &size, (NTAB + 1) * nsl + 2 * (nb + 1));    // slice sizes, the scan's block sums
+    if (e != cudaSuccess) { free_all(tmp); V3_CUDA(e); }
+    const dim3 g((unsigned)blocks_for(q, 128), NTAB);
+    k3_perm<<<blocks_for(q, 256), 256, 0, st>>>(b->N, b->Ni, b->Nb, nsl, nw, b->interior, b->boundary, perm);
+    k3_step_size<<<g, 128, 0, st>>>(A, perm, b->k0, nsl, len, size);
+    int64_t* bsum = reinterpret_cast<int64_t*>(size + ((NTAB + 1) * nsl + 1) / 2 * 2);
+    enqueue_scan(b, size, (NTAB + 1) * nsl, base, bsum);
+    e = cudaMemsetAsync(most, 0, 3 * sizeof(int64_t), st);
+    k3_step_most<<<1, 256, 0, st>>>(nsl, solve_blocks(b), base, (unsigned long long*)most);
+    int64_t h[3] = {0, 0, 0};
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, most, sizeof(h), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    free_all(tmp);
+    V3_CUDA(e);
+    double* val = nullptr;
+    V3_CUDA(alloc(b->build_bufs, &val, h[0] + (h[0] + 1) / 2));            // values, columns
+    int32_t* col = reinterpret_cast<int32_t*>(val + h[0]);
+    k3_step_fill<<<g, 128, 0, st>>>(A, perm, b->k0, nsl, base, col, val);
+    V3_CUDA(cudaGetLastError());
+    for (int t = 0; t < NTAB; ++t) b->tab3[t] = Sell3{base + t * nsl, len + t * q, col, val};
+    b->perm = perm;
+    b->inner = base + NTAB * nsl;
+    b->ent_pois = h[1];
+    b->ent_helm = h[2];
     b->sliced = true;
     return VIP_OK;
 }
@@ -1586,7 +1671,8 @@ vip_status solve_with(vip_3d* b, int kind, double* const* x, int slot) {
     a.alpha = b->dt / (2.0 * b->Re);
     a.rtol = b->rtol;
     a.max_it = b->max_iters;
-    a.t = kind == OPK_HELM ? b->sl_helm : b->sl_pois;
+    a.t = b->tab3[0];
+    a.copied = kind == OPK_HELM ? b->inner : b->tab3[0].base;
     a.ipos = b->ipos;
     a.h = b->h;
     for (int q = 0; q < NS; ++q) {
@@ -1628,29 +1714,28 @@ vip_status solve(vip_3d* b, int kind, double* const* x, int slot) {
 // One fractional step (Eqs. 12-15) on a built node set of interior and wall nodes.
 vip_status step_once(vip_3d* b) {
     const int64_t N = b->N;
-    const unsigned g = blocks_for(N, 128);
+    const unsigned g = blocks_for(32 * b->nsl, 128);
     cudaStream_t st = b->stream;
     const double alpha = b->dt / (2.0 * b->Re), dt = b->dt;
     auto fields = [](double* const* f) { return Fields3{{f[0], f[1], f[2]}}; };
-    const Grad3 G{{b->sl_grad[0], b->sl_grad[1], b->sl_grad[2]}};
-    Vips3 T;
-    for (int k = 0; k < 6; ++k) T.t[k] = b->sl_vip[k];
-    k3_conv<<<g, 128, 0, st>>>(asm_view(b), T, fields(b->vel), fields(b->Ncur));
+    const Asm A = asm_view(b);
+    const Tabs3 T{b->tab3[0], {b->tab3[1], b->tab3[2], b->tab3[3]}, b->perm, 32 * b->nsl, N, b->k0, b->ipos};
+    k3_conv<<<blocks_for(b->Ni, 32), 96, 0, st>>>(A, fields(b->vel), fields(b->Ncur));
     V3_CUDA(cudaGetLastError());
     if (!b->have_prev)
         for (int c = 0; c < 3; ++c)
             V3_CUDA(cudaMemcpyAsync(b->Nprev[c], b->Ncur[c], N * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    k3_rhs<<<g, 128, 0, st>>>(N, b->sl_lap, G, alpha, dt, b->ipos, fields(b->bc), fields(b->vel), fields(b->Ncur),
-                              fields(b->Nprev), b->p, fields(b->rhs), fields(b->star));
+    k3_rhs<<<g, 128, 0, st>>>(T, alpha, dt, fields(b->bc), fields(b->vel), fields(b->Ncur), fields(b->Nprev), b->p,
+                              fields(b->rhs), fields(b->star));
     V3_CUDA(cudaGetLastError());
     V3_CUDA(cudaMemsetAsync(b->dbar, 0, 2 * sizeof(uint32_t), st));
     V3_TRY(solve<3>(b, OPK_HELM, b->star, 0));
     for (int c = 0; c < 3; ++c) std::swap(b->Ncur[c], b->Nprev[c]);
     b->have_prev = true;
-    k3_div<<<g, 128, 0, st>>>(N, G, dt, b->k0, b->ipos, fields(b->star), b->rhs[0]);
+    k3_div<<<g, 128, 0, st>>>(T, dt, fields(b->star), b->rhs[0]);
     V3_CUDA(cudaGetLastError());
     V3_TRY(solve<1>(b, OPK_POIS, &b->phi, 3));
-    k3_project<<<g, 128, 0, st>>>(N, b->sl_lap, G, alpha, dt, b->ipos, b->phi, fields(b->star), fields(b->vel), b->p);
+    k3_project<<<g, 128, 0, st>>>(T, A, alpha, dt, b->phi, fields(b->star), fields(b->vel), b->p);
     V3_CUDA(cudaGetLastError());
     Out3 out[4] = {};
     uint32_t word[2] = {0, 0};
