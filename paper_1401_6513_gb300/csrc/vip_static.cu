@@ -34,9 +34,15 @@ constexpr int NVEC = 6;                      // r, rhat, p, v, s, t
 constexpr int MAX_BLOCKS = 1024;
 constexpr int NQ = 3;                        // reduced quantities per phase, at most
 constexpr int THREADS = 512, WARPS = THREADS / 32;
-// One block up to ONE_BLOCK rows (its barrier is a __syncthreads: 204 rows take 11.5 us per
-// iteration, 15.2 in four blocks), else at least MIN_ROWS rows per block.
+// At least MIN_ROWS rows per block.  Up to ONE_BLOCK rows the first block solves alone if its
+// shared memory holds the matrix (its barrier is a __syncthreads: 204 rows of 5 entries take
+// 11.5 us per iteration, 15.2 in four blocks); 500 rows of 500 entries take 546 us in one block
+// and 157 in eight.  The host does not know the entry count, so the kernel decides.
 constexpr int ONE_BLOCK = 512, MIN_ROWS = 64;
+// Shared memory asked for the matrix up to ONE_BLOCK rows: 32 entries a row, SMALL_MATRIX at
+// least (a dense one of 120 rows in two blocks); a solve of 250 rows leaves half of its SM to
+// others.  Beyond, where every SM has a block, all there is.
+constexpr int64_t SMALL_MATRIX = 96 << 10;
 constexpr int64_t OFF_PART = NVEC * MAX_ROWS;
 // two sets of block partials, used by alternate reductions: a block that runs
 // ahead into the next reduction never overwrites a partial another block is
@@ -108,8 +114,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_bicgstab_static(Args a) {
     __shared__ double red[NQ][THREADS];
     __shared__ double tot[NQ];
     __shared__ Scalars S;
-    const unsigned nb = gridDim.x;
     const int64_t n = a.n;
+    unsigned nb = gridDim.x;
+    if (nb > 1 && n <= ONE_BLOCK && (a.ptr[n] - a.ptr[0]) * 12 + (n + 1) * 8 <= a.mat_smem) {
+        if (blockIdx.x > 0) return;
+        nb = 1;
+    }
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t row0 = n * blockIdx.x / nb;
     const int rows = (int)(n * (blockIdx.x + 1) / nb - row0);
@@ -403,18 +413,18 @@ extern "C" vip_status vip_bicgstab_static(int device, void* cuda_stream, int64_t
     int sms = 0, smem = 0;
     vip_status st0 = setup(device, &ws, &sms, &smem);
     if (st0 != VIP_OK) return st0;
-    const int grid = n <= ONE_BLOCK ? 1
-                                    : (int)std::min<int64_t>({(n + MIN_ROWS - 1) / MIN_ROWS, (int64_t)sms,
-                                                              (int64_t)MAX_BLOCKS});
+    const int grid = (int)std::min<int64_t>({(n + MIN_ROWS - 1) / MIN_ROWS, (int64_t)sms, (int64_t)MAX_BLOCKS});
     Args a{n, row_ptr, col, val, b, x, rtol, max_iters, ws, reinterpret_cast<unsigned int*>(ws + OFF_RES + 4), 0, 0};
-    const int64_t vb = (int64_t)(NVEC + 1) * ((n + grid - 1) / grid) * 8;
+    const int64_t rows = n <= ONE_BLOCK ? n : (n + grid - 1) / grid;   // of a block, at most
+    const int64_t vb = (NVEC + 1) * rows * 8;
     a.vec_smem = vb <= smem;
-    a.mat_smem = smem - (a.vec_smem ? vb : 0);
+    const int64_t dyn = n <= ONE_BLOCK ? std::min<int64_t>(smem, vb + std::max(SMALL_MATRIX, n * 32 * 12)) : smem;
+    a.mat_smem = dyn - (a.vec_smem ? vb : 0);
     // the barrier word and the result record start at zero on every call; the
     // Krylov vectors and partials need no clearing (each is written before it is read)
     if (cudaMemsetAsync(ws + OFF_RES, 0, 8 * sizeof(double), st) != cudaSuccess) return VIP_ERR_CUDA;
     void* args[] = {&a};
-    if (cudaLaunchCooperativeKernel((const void*)k_bicgstab_static, dim3(grid), dim3(THREADS), args, (size_t)smem, st) !=
+    if (cudaLaunchCooperativeKernel((const void*)k_bicgstab_static, dim3(grid), dim3(THREADS), args, (size_t)dyn, st) !=
         cudaSuccess)
         return VIP_ERR_CUDA;
     double h[4] = {0, 0, 0, 0};
