@@ -431,9 +431,7 @@ struct Cnn {
     float* s_dprev = nullptr;       // (phi^n - phi^{n-1}) / S of each sample (FP32)
     // test images (vip_cnn_forward / vip_cnn_grads)
     CnnImage* timg = nullptr;
-    // input of vip_ws_eval (BF16, kept and grown like the activations), count of its loss cells
-    __nv_bfloat16* ein = nullptr;
-    int64_t ein_cells = 0;
+    // count of vip_ws_eval's loss cells
     unsigned long long* ecnt = nullptr;   // [2]: the count, the bits of its reciprocal
 };
 
@@ -1068,12 +1066,8 @@ vip_status vip_ws_eval(vip_ctx* c, int32_t H, int32_t W, const float* x, float* 
     // input: FP32 [H][W][16] -> BF16, read where it lies if that is this device's memory.  Writers
     // of the caller's arrays on the default stream have finished, whatever kind of stream s is.
     VIP_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
-    if (N.ein_cells < n) {
-        VIP_CUDA(dalloc(c, &N.ein, n * CNN_CIN));
-        N.ein_cells = n;
-    }
     if (!N.ecnt) VIP_CUDA(dalloc(c, &N.ecnt, 2));
-    __nv_bfloat16* in = N.ein;
+    __nv_bfloat16* in = N.act[0];   // (a step fills it anew)
     EvalArray dx, dt, dm;
     VIP_CUDA(dx.get(c, x, n * CNN_CIN, s));
     k_ws_input<<<nblk(n * CNN_CIN / 4, 256), 256, 0, s>>>(n * CNN_CIN / 4, reinterpret_cast<const float4*>(dx.p),
