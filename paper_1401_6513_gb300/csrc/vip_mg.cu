@@ -826,27 +826,42 @@ vip_status mg_build(vip_ctx* c, Multigrid& M) {
         VIP_CUDA(cudaMemcpyAsync(M.cinv_off, ioff.data(), G * 8, cudaMemcpyHostToDevice, st));
         std::vector<BandMat> mats;
         std::vector<int2> dims;
+        // small inverses: on the host, each run of neighbouring geometries copied at once
+        std::vector<double> Ad, hinv;
+        std::vector<float> hinv32;
+        int64_t run = 0;   // the run's place in cinv
+        auto flush = [&]() -> vip_status {
+            if (hinv.empty()) return VIP_OK;
+            hinv32.assign(hinv.begin(), hinv.end());
+            VIP_CUDA(cudaMemcpyAsync(M.cinv + run, hinv.data(), hinv.size() * 8, cudaMemcpyHostToDevice, st));
+            VIP_CUDA(cudaMemcpyAsync(M.cinv32 + run, hinv32.data(), hinv32.size() * 4, cudaMemcpyHostToDevice, st));
+            VIP_CUDA(cudaStreamSynchronize(st));
+            hinv.clear();
+            return VIP_OK;
+        };
         for (int g = 0; g < G; ++g) {
             const int m = hg[g].nx[L] * hg[g].ny[L];
             const int64_t c0 = offs[L][g];  // cells numbered densely on the coarsest level
             if (m > HOST_INVERSE) {
                 mats.push_back({0, 0, ioff[g], c0, 0, m, 0, 0});
                 dims.push_back(make_int2(hg[g].nx[L], hg[g].ny[L]));
+                const vip_status s = flush();
+                if (s != VIP_OK) return s;
                 continue;
             }
-            std::vector<double> Ad((size_t)m * m, 0.0), inv((size_t)m * m);
-            std::vector<float> inv32((size_t)m * m);
+            Ad.assign((size_t)m * m, 0.0);
             for (int r = 0; r < m; ++r)
                 for (int o = 0; o < 25; ++o) {
                     const int32_t j = hnbr[(size_t)o * lc.n + c0 + r];
                     if (j >= 0) Ad[(size_t)r * m + (j - c0)] += hcoef[(size_t)o * lc.n + c0 + r];
                 }
-            coarse_inverse(Ad, m, inv.data());
-            for (size_t i = 0; i < inv.size(); ++i) inv32[i] = (float)inv[i];
-            VIP_CUDA(cudaMemcpyAsync(M.cinv + ioff[g], inv.data(), inv.size() * 8, cudaMemcpyHostToDevice, st));
-            VIP_CUDA(cudaMemcpyAsync(M.cinv32 + ioff[g], inv32.data(), inv32.size() * 4, cudaMemcpyHostToDevice,
-                                     st));
-            VIP_CUDA(cudaStreamSynchronize(st));
+            if (hinv.empty()) run = ioff[g];
+            hinv.resize(hinv.size() + (size_t)m * m);
+            coarse_inverse(Ad, m, hinv.data() + (ioff[g] - run));
+        }
+        {
+            const vip_status s = flush();
+            if (s != VIP_OK) return s;
         }
         if (!mats.empty()) {
             const vip_status s = band_inverses(c, M, lc, mats, dims, hnbr.data());
