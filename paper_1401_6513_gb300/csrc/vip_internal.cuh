@@ -109,7 +109,6 @@ struct KrylovPlan {
     int32_t* sys_s0 = nullptr;      // [nsys] slice range of a system
     int32_t* sys_s1 = nullptr;
     double* partial = nullptr;      // [2][nsys][NQ][nblocks]: two sets, alternate reductions
-    int32_t* flags = nullptr;       // [nblocks]
     uint32_t* bar = nullptr;        // [2] barrier count / generation
     // per-system outputs
     int32_t* out_iters = nullptr;

@@ -1552,7 +1552,6 @@ vip_status krylov_plan(vip_ctx* c, KrylovPlan& P, const Sell& A, const std::vect
     // dot-product sums, the coarse tile and the shared stencils live in dynamic shared
     // memory (set here, outside any graph capture); as much L1 as possible for the vector
     // gathers: the smallest shared-memory configuration that holds the block
-    int occ = 1;
     {
         struct { const void* k; int nt, dyn; } kern[] = {
             {(const void*)k_bicgstab<double, double, NT64>, NT64, dyn_bytes<double, double, NT64>()},
@@ -1577,9 +1576,8 @@ vip_status krylov_plan(vip_ctx* c, KrylovPlan& P, const Sell& A, const std::vect
     }
     for (int64_t s = 0; s < nsl; ++s)
         if (slice_sys[s] < 0) { c->err = "slice without system"; return VIP_ERR_ARG; }
-    // contiguous slice chunks, one per block; a block may touch MAXSYS_PB systems
-    int nb = std::max(1, c->num_sms * occ);
-    nb = (int)std::min<int64_t>(nb, nsl);
+    // contiguous slice chunks, one per block (one per SM); a block may touch MAXSYS_PB systems
+    const int nb = (int)std::min<int64_t>(std::max(1, c->num_sms), nsl);
     std::vector<int32_t> bs0(nb), bs1(nb), bg0(nb), bng(nb);
     std::vector<int32_t> sb0(nsys, 1 << 30), sb1(nsys, -1);
     for (int b = 0; b < nb; ++b) {
@@ -1604,7 +1602,6 @@ vip_status krylov_plan(vip_ctx* c, KrylovPlan& P, const Sell& A, const std::vect
     VIP_CUDA(dalloc(c, &P.sys_s0, nsys)); VIP_CUDA(dalloc(c, &P.sys_s1, nsys));
     VIP_CUDA(dalloc(c, &P.partial, (size_t)2 * nb * nsys * NQ));
     VIP_CUDA(cudaMemsetAsync(P.partial, 0, (size_t)2 * nb * nsys * NQ * sizeof(double), c->stream));
-    VIP_CUDA(dalloc(c, &P.flags, nb));
     VIP_CUDA(dalloc(c, &P.bar, 2));
     VIP_CUDA(dalloc(c, &P.out_iters, nsys)); VIP_CUDA(dalloc(c, &P.out_outer, nsys));
     VIP_CUDA(dalloc(c, &P.out_relres, nsys)); VIP_CUDA(dalloc(c, &P.out_status, nsys));

@@ -27,7 +27,7 @@ def forced(request, vip, tmp_path_factory):
     subprocess.run([build.nvcc(), *build.NVCC_FLAGS, *build.ARCH, "-w", *FORMS[request.param], "-I", str(build.CSRC),
                     "-c", str(build.CSRC / "vip_krylov.cu"), "-o", str(d / "k.o")], check=True)
     subprocess.run([build.nvcc(), *build.ARCH, "-shared", "-o", str(d / "libvip_forced.so"), str(d / "k.o"),
-                    *map(str, others), "-lcudart", "-Xcompiler", "-fopenmp"], check=True)
+                    *map(str, others), "-lcudart"], check=True)
     usual, vip._lib = vip._lib, vip.lib(d / "libvip_forced.so")
     yield vip
     vip._lib = usual
