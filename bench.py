@@ -316,7 +316,14 @@ def run_reference(args, rank, ws):
 # launch divided by its inner iterations; profiles/): every iteration streams the same
 # operator and vectors, so a launch's traffic scales with its iterations.  Keyed by
 # workload and form; a form whose kernel changed since its capture has no entry.
-TRAFFIC_PER_ITER = {}
+TRAFFIC_PER_ITER = {
+    # launches of 10 and of 20 iterations: 4.03 and 7.93 GB
+    ("bumpy_h64", "mixed"): 3.90e9 / 10,
+    # 9.12 and 18.04 GB
+    ("bumpy_h64", "fp64"): 8.92e9 / 10,
+    # one launch of 20 iterations, whose working set fits in L2
+    ("cylinder_h32", "mixed"): 72.7e6 / 20,
+}
 
 # FP64 operations per clock per SM of GB300 (two FP64 FMAs), for the ALU roofline;
 # 152 SMs at 2070 MHz give 1.26 TFLOP/s, the part's nominal FP64 rate.

@@ -14,8 +14,10 @@
  *   - Array arguments are plain pointers.  Unless stated otherwise a pointer
  *     may be host memory (pageable or pinned) or device memory of the
  *     context's device; the library copies from / into it (cudaMemcpyDefault).
- *     Inputs are copied, so the caller keeps ownership and may reuse them as
- *     soon as the call returns.  Outputs go into caller-owned buffers.
+ *     Inputs are copied, or (vip_apply, vip_3d_apply, vip_ws_eval: arrays in this
+ *     device's memory) read in place by kernels that have finished when the call
+ *     returns, so the caller keeps ownership and may reuse them then.  Outputs go
+ *     into caller-owned buffers.
  *   - Node arrays are in the caller's order, geometries concatenated in the
  *     order they were added ("global node order").
  *   - Work is issued on the stream passed to vip_create.  Calls that return

@@ -250,7 +250,8 @@ __global__ void k_band_fill(const BandMat* __restrict__ mats, int64_t ncell, con
     if (empty) col[j] = 1.0;
 }
 
-// Band LU with partial pivoting, one block per geometry.  At step k every warp exchanges rows
+// Band LU with partial pivoting (Golub and Van Loan, Matrix Computations, Sec. 4.3; the band
+// with b further diagonals for the fill of row exchanges), one block per geometry.  At step k every warp exchanges rows
 // k and p of its columns and subtracts the multiples of row k from the b rows below; warp 0
 // takes column k + 1 alone, then looks for its pivot and scales it, so that a step needs one
 // barrier and the search and the division run beside the update.  ju is the last column that
@@ -314,7 +315,7 @@ __global__ void __launch_bounds__(512) k_band_factor(const BandMat* __restrict__
             // columns k + 2 .. ju, split over warps 1 .. 15; a warp's columns as one list of elements
             const int nc = ju - k - 1, per = (nc + 14) / 15;
             const int j0 = k + 2 + (warp - 1) * per, jn = min(per, ju + 1 - j0);
-            for (int q0 = 0; q0 < jn; q0 += 32) {      // 32 columns at a time (one, unless b > 160)
+            for (int q0 = 0; q0 < jn; q0 += 32) {      // 32 columns at a time (one pass, unless b > 240)
                 const int qn = min(32, jn - q0);
                 double c = 0.0;
                 if (lane < qn) {
@@ -805,7 +806,7 @@ vip_status mg_build(vip_ctx* c, Multigrid& M) {
             VIP_CUDA(cudaGetLastError());
         }
     }
-    {   // exact solve on the coarsest level: dense inverses, one per geometry (host)
+    {   // exact solve on the coarsest level: dense inverses, one per geometry
         MgLevel& lc = M.lev[L];
         std::vector<int64_t> ioff(G);
         int64_t tot = 0;
